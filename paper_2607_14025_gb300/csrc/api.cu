@@ -438,7 +438,7 @@ void wdf_destroy(wdf_ctx *c) {
   if (c->st) (void)cudaStreamSynchronize(c->st);
   else (void)cudaDeviceSynchronize();
   DBuf *bufs[] = {&c->t_col_off, &c->t_col_zlo, &c->t_e_col, &c->t_e_z,   &c->t_tile,  &c->t_xact,   &c->t_pos3,   &c->t_g2,
-                  &c->t_vhalf,   &c->t_emap,    &c->t_emap2, &c->t_econj, &c->t_tw64,  &c->t_tw32,   &c->vloc64,   &c->vloc32,
+                  &c->t_vhalf,   &c->t_emap,    &c->t_emap2, &c->t_econj, &c->t_tw64,  &c->t_tw32,   &c->vloc64,   &c->vloc32,   &c->vgroup32,
                   &c->U64,       &c->U32,       &c->lrd,     &c->psir64,  &c->psir32,  &c->kp64,     &c->kp32,     &c->tkin,
                   &c->eps_dev,   &c->rb,        &c->rx,      &c->rr,      &c->rAx,     &c->rwork,    &c->shift,    &c->vidx_dev,
                   &c->thr,       &c->gramw,     &c->xpert,   &c->dvgrid,  &c->accgrid, &c->cb2,      &c->outi,     &c->drhoi,

