@@ -227,6 +227,7 @@ __global__ void k_sum_splits(const double *__restrict__ part, int nsplit, size_t
   if (t >= na * nb) return;
   const int i = t / nb, j = t % nb;
   double s = 0.0;
+#pragma unroll 8
   for (int z = 0; z < nsplit; ++z) s += part[z * stride + (size_t)i * ldo + j];
   out[(size_t)i * ldo + j] = s;
 }
@@ -262,6 +263,98 @@ __global__ void __launch_bounds__(256) k_gram_narrow(Geo g, const cplx<T> *__res
   }
 }
 
+// FP64 Gram products with more than 8 right-hand vectors. The FP64 pipe does 2 FMAs per clock and SM
+// (1.19 TFLOP/s in all), so an FMA instruction of a warp takes 16 clocks and feeding it costs
+// nothing: what matters is that no FMA is spent on padding and that every SM has its share. Output
+// tiles of 16 x 16 (2 x 4 per lane), the four warps of a block taking every fourth chunk of GE64
+// elements of the block's K range and adding up in shared memory, K split over blocks so that the
+// last wave is full (gram_split_f64). Against the 64 x 128 tile of k_gram (one GB300, 8,455
+// elements): 128 x 48 outputs 0.98 -> 0.24 ms, 64 x 47 0.98 -> 0.13 ms (FMA floors 0.17 and 0.085 ms);
+// 42 x 56 of 1,800 elements 0.22 -> 0.021 ms.
+constexpr int GT64 = 16;
+constexpr int GE64 = 8;
+
+__global__ void __launch_bounds__(128) k_gram_f64(Geo g, const double2 *__restrict__ A, int na, const double2 *__restrict__ B, int nb,
+                                                 double *__restrict__ out, int ldo, int echunk, size_t split_stride) {
+  __shared__ double2 As[4][GE64][GT64 + 1], Bs[4][GE64][GT64 + 1];
+  __shared__ double red[3][GT64 * GT64];
+  const int j0 = blockIdx.x * GT64, i0 = blockIdx.y * GT64;
+  const int ebeg = blockIdx.z * echunk, eend = min(g.nint, ebeg + echunk);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, ty = lane >> 2, tx = lane & 3;
+  double acc[2][4];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
+  for (int e0 = ebeg + w * GE64; e0 < eend; e0 += 4 * GE64) {
+    double2 ra[4], rb[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {  // 8 consecutive lanes read 8 consecutive elements of a row
+      const int row = (lane >> 3) + 4 * u, e = e0 + (lane & 7);
+      ra[u] = rb[u] = make_double2(0.0, 0.0);
+      if (e < eend && i0 + row < na) {
+        ra[u] = A[(size_t)(i0 + row) * g.ld + e];
+        const double wt = wgt(e, g.len0);
+        ra[u].x *= wt;
+        ra[u].y *= wt;
+      }
+      if (e < eend && j0 + row < nb) rb[u] = B[(size_t)(j0 + row) * g.ld + e];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      As[w][lane & 7][(lane >> 3) + 4 * u] = ra[u];
+      Bs[w][lane & 7][(lane >> 3) + 4 * u] = rb[u];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < GE64; ++k) {
+      double2 av[2], bv[4];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) av[a] = As[w][k][ty + 8 * a];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) bv[b] = Bs[w][k][tx + 4 * b];
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a].x, bv[b].x, fma(av[a].y, bv[b].y, acc[a][b]));
+    }
+  }
+  if (w > 0)
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) red[w - 1][(ty + 8 * a) * GT64 + tx + 4 * b] = acc[a][b];
+  __syncthreads();
+  if (w > 0) return;
+  double *o = out + blockIdx.z * split_stride;
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int r = ty + 8 * a, c = tx + 4 * b, i = i0 + r, j = j0 + c;
+      const double v = ((acc[a][b] + red[0][r * GT64 + c]) + red[1][r * GT64 + c]) + red[2][r * GT64 + c];
+      if (i < na && j < nb) o[(size_t)i * ldo + j] = v;
+    }
+}
+
+// K splits (at most 64) and elements per split of k_gram_f64: the fewest whole waves of blocks times
+// their length, a block counted as its elements plus the 48 that its start and sums take
+static int gram_split_f64(const Geo &g, int na, int nb, int &echunk) {
+  const long tiles = (long)((na + GT64 - 1) / GT64) * ((nb + GT64 - 1) / GT64);
+  const int unit = 4 * GE64;
+  long best = -1;
+  for (int s = 1; s <= 64; ++s) {
+    const int ec = ((g.nint + s - 1) / s + unit - 1) / unit * unit, ns = (g.nint + ec - 1) / ec;
+    const long cost = (tiles * ns + 151) / 152 * (ec + 48) + 4L * ns;
+    if (best < 0 || cost < best) {
+      best = cost;
+      echunk = ec;
+    }
+  }
+  return (g.nint + echunk - 1) / echunk;
+}
+
 static int gram_nsplit(const Geo &g, int na, int nb, int &echunk) {
   const int tiles = ((na + GI - 1) / GI) * ((nb + GJ - 1) / GJ);
   int nsplit = 1;
@@ -278,22 +371,35 @@ static int gram_nsplit(const Geo &g, int na, int nb, int &echunk) {
 
 size_t gram_work_doubles(const Geo &g, int na, int nb, int ldo) {
   int echunk;
-  const int nsplit = gram_nsplit(g, na, nb, echunk);
+  int nsplit = gram_nsplit(g, na, nb, echunk);
+  if (nb > kNarrow) nsplit = std::max(nsplit, gram_split_f64(g, na, nb, echunk));
   return nsplit > 1 ? (size_t)na * ldo * nsplit : 0;
 }
 
 // Split over elements when the output has too few tiles to fill the GPU; the partial sums go to
 // work (caller-owned, gram_work_doubles() long) and are added in a fixed order.
-template <typename T>
-void launch_gram(const Geo &g, const cplx<T> *A, int na, const cplx<T> *B, int nb, double *out, int ldo, double *work,
-                 size_t work_cap, cudaStream_t st) {
-  if (na <= 0 || nb <= 0) return;
-  typedef typename std::conditional<std::is_same<T, float>::value, float, T>::type AccN;
-  if (nb <= kNarrow) {
-    launch("gram", bits_of<T>(), k_gram_narrow<T, AccN>, dim3(na), dim3(256), 0, st, g, A, B, nb, out, ldo);
-    WDF_CUDA_TRY(cudaGetLastError());
-    return;
+static void launch_gram_f64(const Geo &g, const double2 *A, int na, const double2 *B, int nb, double *out, int ldo, double *work,
+                            size_t work_cap, cudaStream_t st) {
+  int echunk;
+  int nsplit = gram_split_f64(g, na, nb, echunk);
+  const size_t stride = (size_t)na * ldo;
+  if (nsplit > 1 && (work == nullptr || work_cap < stride * nsplit)) {
+    nsplit = 1;
+    echunk = g.nint;
   }
+  launch("gram", 64, k_gram_f64, dim3((nb + GT64 - 1) / GT64, (na + GT64 - 1) / GT64, nsplit), dim3(128), 0, st, g, A, na, B, nb,
+         nsplit > 1 ? work : out, ldo, echunk, nsplit > 1 ? stride : (size_t)0);
+  WDF_CUDA_TRY(cudaGetLastError());
+  if (nsplit > 1) {
+    launch("gram_sum", 0, k_sum_splits, dim3((na * nb + 255) / 256), dim3(256), 0, st, (const double *)work, nsplit, stride, out, na, nb, ldo);
+    WDF_CUDA_TRY(cudaGetLastError());
+  }
+}
+
+// FP32 and double-float
+template <typename T>
+static void launch_gram_wide(const Geo &g, const cplx<T> *A, int na, const cplx<T> *B, int nb, double *out, int ldo, double *work,
+                             size_t work_cap, cudaStream_t st) {
   int echunk;
   int nsplit = gram_nsplit(g, na, nb, echunk);
   const size_t stride = (size_t)na * ldo;
@@ -302,28 +408,34 @@ void launch_gram(const Geo &g, const cplx<T> *A, int na, const cplx<T> *B, int n
     echunk = ((g.nint + GK - 1) / GK) * GK;
   }
   dim3 grid((na + GI - 1) / GI, (nb + GJ - 1) / GJ, nsplit);
-  typedef typename std::conditional<std::is_same<T, float>::value, float, T>::type Acc;  // T for FP64 and double-float
   if constexpr (std::is_same<T, float>::value) {
     echunk = ((echunk + GK32 - 1) / GK32) * GK32;  // whole 32-element chunks per split
     grid.z = nsplit = (g.nint + echunk - 1) / echunk;
-    if (nsplit == 1) {
-      launch("gram", 32, k_gram_f32, dim3(grid), dim3(256), 0, st, g, A, na, B, nb, out, ldo, echunk, (size_t)0);
-    } else {
-      launch("gram", 32, k_gram_f32, dim3(grid), dim3(256), 0, st, g, A, na, B, nb, work, ldo, echunk, stride);
-      WDF_CUDA_TRY(cudaGetLastError());
-      launch("gram_sum", 0, k_sum_splits, dim3((na * nb + 255) / 256), dim3(256), 0, st, work, nsplit, stride, out, na, nb, ldo);
-    }
-    WDF_CUDA_TRY(cudaGetLastError());
-    return;
-  }
-  if (nsplit == 1) {
-    launch("gram", bits_of<T>(), k_gram<T, Acc>, dim3(grid), dim3(256), 0, st, g, A, na, B, nb, out, ldo, echunk, 0);
+    launch("gram", 32, k_gram_f32, grid, dim3(256), 0, st, g, A, na, B, nb, nsplit > 1 ? work : out, ldo, echunk,
+           nsplit > 1 ? stride : (size_t)0);
   } else {
-    launch("gram", bits_of<T>(), k_gram<T, Acc>, dim3(grid), dim3(256), 0, st, g, A, na, B, nb, work, ldo, echunk, stride);
-    WDF_CUDA_TRY(cudaGetLastError());
-    launch("gram_sum", 0, k_sum_splits, dim3((na * nb + 255) / 256), dim3(256), 0, st, work, nsplit, stride, out, na, nb, ldo);
+    launch("gram", bits_of<T>(), k_gram<T, T>, grid, dim3(256), 0, st, g, A, na, B, nb, nsplit > 1 ? work : out, ldo, echunk,
+           nsplit > 1 ? stride : (size_t)0);
   }
   WDF_CUDA_TRY(cudaGetLastError());
+  if (nsplit > 1) {
+    launch("gram_sum", 0, k_sum_splits, dim3((na * nb + 255) / 256), dim3(256), 0, st, (const double *)work, nsplit, stride, out, na, nb, ldo);
+    WDF_CUDA_TRY(cudaGetLastError());
+  }
+}
+
+template <typename T>
+void launch_gram(const Geo &g, const cplx<T> *A, int na, const cplx<T> *B, int nb, double *out, int ldo, double *work,
+                 size_t work_cap, cudaStream_t st) {
+  if (na <= 0 || nb <= 0) return;
+  if (nb <= kNarrow) {
+    launch("gram", bits_of<T>(), k_gram_narrow<T, T>, dim3(na), dim3(256), 0, st, g, A, B, nb, out, ldo);
+    WDF_CUDA_TRY(cudaGetLastError());
+  } else if constexpr (std::is_same<T, double>::value) {
+    launch_gram_f64(g, A, na, B, nb, out, ldo, work, work_cap, st);
+  } else {
+    launch_gram_wide<T>(g, A, na, B, nb, out, ldo, work, work_cap, st);
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -432,6 +544,86 @@ __global__ void __launch_bounds__(256) k_lincomb(Geo g, cplx<T> *__restrict__ Y,
   }
 }
 
+// FP64 linear combinations into more than 8 vectors: a warp owns 32 elements (a block LE = 128) of VQ
+// vectors, each lane one element, rows of U read once per VQ vectors (coalesced, from L2), the
+// scaled coefficients staged LJ64 rows at a time. As for the Gram products only the FMAs count: at
+// most VQ - 1 padded vectors and enough blocks for the 152 SMs. VQ = 4 until the vectors alone
+// make two blocks per SM with 8. Against the 128 x 32 tile of k_lincomb: 42 rows into 56 vectors of
+// 1,800 elements 97 -> 20 us, 128 rows into 48 of 8,455 278 -> 201 us, 64 into 47 138 -> 101 us.
+constexpr int LJ64 = 64;
+
+template <int VQ>
+__global__ void __launch_bounds__(128) k_lincomb_f64(Geo g, double2 *__restrict__ Y, int ny, const double2 *__restrict__ U, int nu,
+                                                    const double *__restrict__ C, int ldc, const double *__restrict__ d, double c0,
+                                                    const double2 *__restrict__ P, double *__restrict__ part) {
+  __shared__ double cs[LJ64][VQ];
+  __shared__ double red[4][VQ];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int s0 = blockIdx.x * VQ, e = blockIdx.y * LE + threadIdx.x;
+  const bool on = e < g.nint;
+  double ax[VQ], ay[VQ];
+#pragma unroll
+  for (int q = 0; q < VQ; ++q) ax[q] = ay[q] = 0.0;
+  for (int j0 = 0; j0 < nu; j0 += LJ64) {
+    const int jn = min(LJ64, nu - j0);
+    for (int t = threadIdx.x; t < jn * VQ; t += 128) {
+      const int j = j0 + t / VQ, s = s0 + t % VQ;
+      cs[t / VQ][t % VQ] = s < ny ? C[(size_t)j * ldc + s] * (d ? d[j] : 1.0) : 0.0;
+    }
+    __syncthreads();
+    const double2 *u = U + (size_t)j0 * g.ld + e;
+#pragma unroll 4
+    for (int jj = 0; jj < jn; ++jj) {
+      const double2 uv = on ? u[(size_t)jj * g.ld] : make_double2(0.0, 0.0);
+#pragma unroll
+      for (int q = 0; q < VQ; ++q) {
+        const double c = cs[jj][q];
+        ax[q] = fma(c, uv.x, ax[q]);
+        ay[q] = fma(c, uv.y, ay[q]);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < VQ; ++q) {
+    const int s = s0 + q;
+    double dsum = 0.0;
+    if (on && s < ny) {
+      double2 *y = Y + (size_t)s * g.ld + e;
+      double2 yv = make_double2(ax[q], ay[q]);
+      if (c0 != 0.0) {
+        const double2 o = *y;
+        yv = make_double2(c0 * o.x + ax[q], c0 * o.y + ay[q]);
+      }
+      *y = yv;
+      if (part) {
+        const double2 pv = P[(size_t)s * g.ld + e];
+        dsum = wgt(e, g.len0) * (pv.x * yv.x + pv.y * yv.y);
+      }
+    }
+    if (part) {
+      for (int o = 16; o > 0; o >>= 1) dsum += __shfl_down_sync(0xffffffffu, dsum, o);
+      if (lane == 0) red[w][q] = dsum;
+    }
+  }
+  if (part == nullptr) return;
+  __syncthreads();
+  if (threadIdx.x < VQ && s0 + threadIdx.x < ny) {
+    const int q = threadIdx.x;
+    part[(size_t)(s0 + q) * gridDim.y + blockIdx.y] = ((red[0][q] + red[1][q]) + red[2][q]) + red[3][q];
+  }
+}
+
+static void launch_lincomb_f64(const Geo &g, double2 *Y, int ny, const double2 *U, int nu, const double *C, int ldc, const double *d,
+                               double c0, const double2 *P, double *part, cudaStream_t st) {
+  const int ne = (g.nint + LE - 1) / LE;
+  if ((long)ne * ((ny + 7) / 8) >= 4 * 152)
+    launch("lincomb", 64, k_lincomb_f64<8>, dim3((ny + 7) / 8, ne), dim3(128), 0, st, g, Y, ny, U, nu, C, ldc, d, c0, P, part);
+  else
+    launch("lincomb", 64, k_lincomb_f64<4>, dim3((ny + 3) / 4, ne), dim3(128), 0, st, g, Y, ny, U, nu, C, ldc, d, c0, P, part);
+  WDF_CUDA_TRY(cudaGetLastError());
+}
+
 // Linear combinations into at most 8 vectors: each thread owns one element of every output.
 template <typename T, typename Acc>
 __global__ void __launch_bounds__(256) k_lincomb_narrow(Geo g, cplx<T> *__restrict__ Y, int ny, const cplx<T> *__restrict__ U, int nu,
@@ -476,11 +668,14 @@ void launch_lincomb(const Geo &g, cplx<T> *Y, int ny, const cplx<T> *U, int nu, 
     WDF_CUDA_TRY(cudaGetLastError());
     return;
   }
-  dim3 grid((g.nint + LE - 1) / LE, (ny + LS - 1) / LS);
-  typedef typename std::conditional<std::is_same<T, float>::value, float, T>::type Acc;  // T for FP64 and double-float
-  launch("lincomb", bits_of<T>(), k_lincomb<T, Acc>, dim3(grid), dim3(256), 0, st, g, Y, ny, U, nu, C, ldc, d, c0,
-         (const cplx<T> *)nullptr, (double *)nullptr);
-  WDF_CUDA_TRY(cudaGetLastError());
+  if constexpr (std::is_same<T, double>::value) {
+    launch_lincomb_f64(g, Y, ny, U, nu, C, ldc, d, c0, nullptr, nullptr, st);
+  } else {
+    dim3 grid((g.nint + LE - 1) / LE, (ny + LS - 1) / LS);
+    launch("lincomb", bits_of<T>(), k_lincomb<T, T>, dim3(grid), dim3(256), 0, st, g, Y, ny, U, nu, C, ldc, d, c0,
+           (const cplx<T> *)nullptr, (double *)nullptr);
+    WDF_CUDA_TRY(cudaGetLastError());
+  }
 }
 
 int lincomb_dot_chunks(const Geo &g) { return (g.nint + LE - 1) / LE; }
@@ -489,10 +684,13 @@ template <typename T>
 bool launch_lincomb_dot(const Geo &g, cplx<T> *Y, int ny, const cplx<T> *U, int nu, const double *C, int ldc, const double *d,
                         double c0, const cplx<T> *P, double *part, cudaStream_t st) {
   if (ny <= kNarrow) return false;  // the narrow kernel has no dot epilogue
-  dim3 grid((g.nint + LE - 1) / LE, (ny + LS - 1) / LS);
-  typedef typename std::conditional<std::is_same<T, float>::value, float, T>::type Acc;
-  launch("lincomb", bits_of<T>(), k_lincomb<T, Acc>, dim3(grid), dim3(256), 0, st, g, Y, ny, U, nu, C, ldc, d, c0, P, part);
-  WDF_CUDA_TRY(cudaGetLastError());
+  if constexpr (std::is_same<T, double>::value) {
+    launch_lincomb_f64(g, Y, ny, U, nu, C, ldc, d, c0, P, part, st);
+  } else {
+    dim3 grid((g.nint + LE - 1) / LE, (ny + LS - 1) / LS);
+    launch("lincomb", bits_of<T>(), k_lincomb<T, T>, dim3(grid), dim3(256), 0, st, g, Y, ny, U, nu, C, ldc, d, c0, P, part);
+    WDF_CUDA_TRY(cudaGetLastError());
+  }
   return true;
 }
 
