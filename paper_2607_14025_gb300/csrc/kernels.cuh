@@ -80,9 +80,10 @@ void set_plane_more_limits_df_b(const Geo &g);
 // V_loc for the FP32 line-resident kernels: [z][x / G][y][G], G = 4, 2 or 1 (what divides n1)
 void launch_lines_group_vloc(const Geo &g, const float *v, float *out, cudaStream_t st);
 // line-resident plane kernels (plane_lines*.cu), one size group per translation unit: float V_loc,
-// double-float V_loc, G2R and product; false when the size is not in the group
+// double-float and FP64 V_loc, G2R and product; false when the size is not in the group
 #define WDF_LINES_GROUPS_F32(X) X(lines_f32_a) X(lines_f32_b) X(lines_f32_c)
 #define WDF_LINES_GROUPS_DF(X) X(lines_df_a) X(lines_df_b) X(lines_df_c) X(lines_df_d) X(lines_df_e) X(lines_df_f)
+#define WDF_LINES_GROUPS_F64(X) X(lines_f64_a) X(lines_f64_b) X(lines_f64_c) X(lines_f64_d)
 #define X(NAME)                                                                                      \
   bool launch_##NAME(const FftCtx<float> &f, int op, int nblk, const PlaneArgs<float> &pa, cudaStream_t st); \
   void set_##NAME##_limits(const Geo &g);
@@ -92,6 +93,11 @@ WDF_LINES_GROUPS_F32(X)
   bool launch_##NAME(const FftCtx<df64> &f, int op, int nblk, const PlaneArgs<df64> &pa, cudaStream_t st); \
   void set_##NAME##_limits(const Geo &g);
 WDF_LINES_GROUPS_DF(X)
+#undef X
+#define X(NAME)                                                                                      \
+  bool launch_##NAME(const FftCtx<double> &f, int op, int nblk, const PlaneArgs<double> &pa, cudaStream_t st); \
+  void set_##NAME##_limits(const Geo &g);
+WDF_LINES_GROUPS_F64(X)
 #undef X
 // double-float 64 x 64 plane kernel (plane_df.cu) for OP_VLOC, OP_PROD_R2G and OP_ACCUM
 bool plane_df_available(const Geo &g, const int *jidx);

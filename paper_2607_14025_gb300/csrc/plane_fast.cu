@@ -344,14 +344,21 @@ template <typename T> static void set_lines_limits(const Geo &g) {
     WDF_LINES_GROUPS_F32(X)
   } else if constexpr (std::is_same<T, df64>::value) {
     WDF_LINES_GROUPS_DF(X)
+  } else {
+    WDF_LINES_GROUPS_F64(X)
   }
 #undef X
+}
+// the line-resident kernel runs this context's plane operations: chosen by the setup timing, or FP64
+// without a timing of its own (the ground state, and H x in a double-float context)
+template <typename T> static bool lines_chosen(const FftCtx<T> &f) {
+  return f.vloc_variant == 8 || (std::is_same<T, double>::value && f.vloc_variant == 0 && lines_available(f.g, f.jidx));
 }
 template <typename T> static bool launch_lines(const FftCtx<T> &f, int op, int nblk, const PlaneArgs<T> &pa, cudaStream_t st) {
 #define X(NAME) launch_##NAME(f, op, nblk, pa, st) ||
   if constexpr (std::is_same<T, float>::value) return op == OP_VLOC && (WDF_LINES_GROUPS_F32(X) false);
   else if constexpr (std::is_same<T, df64>::value) return op != OP_ACCUM && (WDF_LINES_GROUPS_DF(X) false);
-  else return false;
+  else return op != OP_ACCUM && (WDF_LINES_GROUPS_F64(X) false);
 #undef X
 }
 
@@ -401,7 +408,7 @@ template <typename T> bool launch_plane_fast(const FftCtx<T> &f, int op, int nbl
   // double-float kernel above, stays on the generic kernel
   if (op == OP_ACCUM || f.jidx == nullptr) return false;
   if (v == 3) return false;
-  if (f.vloc_variant == 8 && launch_lines<T>(f, op, nblk, pa, st)) return true;
+  if (lines_chosen(f) && launch_lines<T>(f, op, nblk, pa, st)) return true;
   // the other plane operations follow the setup timing of the V_loc product: where the generic
   // kernel won it (large double-float planes), they use the generic kernel too
   if (op != OP_VLOC && f.vloc_variant == 3) return false;
@@ -432,7 +439,7 @@ template <typename T> bool plane_variant_available(const FftCtx<T> &f, int v) {
   if (v == 4) return std::is_same<T, float>::value && reg_plane_enabled() && g.n1 == 64 && g.n2 == 64;
   if (v == 5) return std::is_same<T, float>::value && plane_pipe_available(g, f.err);
   if (v == 7) return std::is_same<T, float>::value && plane_pipe2_available(g, f.err);
-  if (v == 8) return (std::is_same<T, df64>::value || (std::is_same<T, float>::value && f.vgroup)) && lines_available(g, f.jidx);
+  if (v == 8) return (!std::is_same<T, float>::value || f.vgroup) && lines_available(g, f.jidx);
   if (v == 6) return std::is_same<T, df64>::value && plane_df_available(g, f.jidx);
   if (v == 2) return plane_fast_supported(g.n1, g.n2) || (!std::is_same<T, double>::value && plane_more_supported(g.n1, g.n2));
   if (v == 1 && std::is_same<T, float>::value && reg_plane_enabled() && g.n1 == g.n2) {
@@ -456,7 +463,7 @@ template <typename T> bool plane_accum_by_g2r(const FftCtx<T> &f) {
     if (f.jidx == nullptr || f.vloc_variant == 3) return false;
     if constexpr (std::is_same<T, df64>::value)
       if (plane_df_available(f.g, f.jidx)) return false;
-    if (f.vloc_variant == 8) return true;
+    if (lines_chosen(f)) return true;
     return plane_fast_supported(f.g.n1, f.g.n2) || (!std::is_same<T, double>::value && plane_more_supported(f.g.n1, f.g.n2));
   }
 }

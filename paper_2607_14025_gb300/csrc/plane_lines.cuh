@@ -68,6 +68,21 @@ WDF_LINES(df64, 72, 3, 1, 4, 3, 4)
 WDF_LINES(df64, 75, 5, 1, 7, 2, 3)
 WDF_LINES(df64, 80, 4, 1, 5, 2, 5)
 WDF_LINES(df64, 96, 4, 1, 6, 2, 3)
+WDF_LINES(double, 24, 1, 8, 3, 4, 1)
+WDF_LINES(double, 30, 1, 6, 3, 3, 1)
+WDF_LINES(double, 32, 2, 3, 3, 5, 2)
+WDF_LINES(double, 36, 2, 4, 5, 3, 3)
+WDF_LINES(double, 40, 2, 4, 5, 2, 2)
+WDF_LINES(double, 45, 3, 2, 5, 3, 5)
+WDF_LINES(double, 48, 2, 2, 3, 4, 4)
+WDF_LINES(double, 50, 5, 2, 9, 2, 2)
+WDF_LINES(double, 54, 3, 1, 3, 4, 3)
+WDF_LINES(double, 60, 2, 1, 2, 4, 3)
+WDF_LINES(double, 64, 4, 1, 4, 4, 2)
+WDF_LINES(double, 72, 3, 1, 4, 2, 4)
+WDF_LINES(double, 75, 5, 1, 7, 2, 3)
+WDF_LINES(double, 80, 4, 1, 5, 2, 5)
+WDF_LINES(double, 96, 4, 1, 6, 2, 3)
 #undef WDF_LINES
 
 // Padding of the exchange buffer: line l, source s, slot a of a chunk sits at l PL + s QS + a. A
@@ -232,22 +247,22 @@ template <typename T, int E, int N> __device__ __forceinline__ void load_run(T (
 
 template <typename T, int N, int OP>
 __global__ void __launch_bounds__(32 * Lines<T, N>::W, Lines<T, N>::B)
-    k_plane_lines(Geo g, const cplx<T> *__restrict__ twg, const int *__restrict__ jidx, PlaneArgs<T> pa, int nunits) {
+    k_plane_lines(Geo g, const cplx<T> *__restrict__ twg, const int *__restrict__ jidx, PlaneArgs<T> pa, int nunits, int ppb) {
   typedef LineXf<T, N> X;
   typedef ld::CA<T> O;
   typedef typename O::C Cx;
   typedef cplx<T> Gx;  // in global memory
   constexpr int L = X::L, M = X::M, KI = X::KI, LW = X::LW, XB = X::XB;
-  constexpr int P = Lines<T, N>::P, W = Lines<T, N>::W, PITCH = 2 * XB + 1, TH = 32 * W;
+  constexpr int W = Lines<T, N>::W, PITCH = 2 * XB + 1, TH = 32 * W;
   constexpr bool STAGE = std::is_same<T, float>::value;  // column-buffer slices through shared memory
   extern __shared__ __align__(16) unsigned char smraw[];
   Cx *tw = reinterpret_cast<Cx *>(smraw);
   Cx *exb = tw + (L > 1 ? N : 0);
   Cx *tile = exb + (L > 1 ? W * X::Pad::size : 0);
-  Gx *slice = reinterpret_cast<Gx *>(tile + P * N * PITCH);
+  Gx *slice = reinterpret_cast<Gx *>((reinterpret_cast<uintptr_t>(tile + ppb * N * PITCH) + 15) & ~(uintptr_t)15);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int nx = g.nxact, xmax = g.xmax, ldcb = g.ldcb;
-  const int u0 = blockIdx.x * P, np = min(P, nunits - u0);
+  const int u0 = blockIdx.x * ppb, np = min(ppb, nunits - u0);
   Gx *cb = pa.cb + (size_t)u0 * ldcb;
   if constexpr (L > 1)
     for (int i = t; i < N; i += TH) tw[i] = O::get(twg[i]);
@@ -374,18 +389,18 @@ __global__ void __launch_bounds__(32 * Lines<T, N>::W, Lines<T, N>::B)
   }
 }
 
-template <typename T, int N> size_t lines_smem(const Geo &g) {
+template <typename T, int N> size_t lines_smem(const Geo &g, int ppb) {
   typedef LineXf<T, N> X;
   typedef Lines<T, N> D;
-  size_t n = (size_t)D::P * N * (2 * (N / 4) + 1);
+  size_t n = (size_t)ppb * N * (2 * (N / 4) + 1);
   if (D::L > 1) n += N + (size_t)D::W * X::Pad::size;
-  if (std::is_same<T, float>::value) n += (size_t)D::P * g.ldcb;
-  return n * sizeof(cplx<T>);
+  if (std::is_same<T, float>::value) n += (size_t)ppb * g.ldcb;
+  return n * sizeof(cplx<T>) + 16;  // 16: the slices of an odd tile start on the next 16 bytes
 }
 
 template <typename T, int N> void lines_limits_n(const Geo &g) {
   if (g.n1 != N || g.n2 != N) return;
-  const size_t sm = lines_smem<T, N>(g);
+  const size_t sm = lines_smem<T, N>(g, Lines<T, N>::P);
   if (sm > 227 * 1024) return;
   raise_smem_limit(k_plane_lines<T, N, OP_VLOC>, sm);
   if constexpr (!std::is_same<T, float>::value) {
@@ -400,9 +415,12 @@ void lines_launch_op(const char *cls, const FftCtx<T> &f, int npair, const Plane
   const int nunits = npair * f.g.n3;
   PlaneArgs<T> a = pa;
   if (std::is_same<T, float>::value) a.field = f.vgroup;
-  const dim3 grid((unsigned)((nunits + D::P - 1) / D::P));
-  launch_units(cls, bits_of<T>(), nunits, k_plane_lines<T, N, OP>, grid, dim3(32 * D::W), lines_smem<T, N>(f.g), st, f.g, f.tw1, f.jidx,
-               a, nunits);
+  // few units: fewer planes per block, so that every SM has its blocks before a block has a second
+  // plane (8 solves on 24 x 24: 96 units, 12 blocks of 8 planes against 96 of one)
+  const int ppb = std::max(1, std::min(D::P, (nunits + 152 * D::B - 1) / (152 * D::B)));
+  const dim3 grid((unsigned)((nunits + ppb - 1) / ppb));
+  launch_units(cls, bits_of<T>(), nunits, k_plane_lines<T, N, OP>, grid, dim3(32 * D::W), lines_smem<T, N>(f.g, ppb), st, f.g, f.tw1, f.jidx,
+               a, nunits, ppb);
   WDF_CUDA_TRY(cudaGetLastError());
 }
 

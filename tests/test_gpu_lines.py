@@ -77,6 +77,24 @@ def test_operator_and_response_match_the_generic_kernel(n, nvec):
     assert abs(a[3] - b[3]) <= max(2, 0.03 * b[3])
 
 
+@pytest.mark.parametrize("n", synth.GRID_SIZES)
+def test_fp64_form_matches_the_generic_kernel(n):
+    """FP64: both within a few ulp (1e-16 of the largest value per transform); bar 1e-14."""
+    s = probe(n)
+    psi = synth.make_guess(s, s.nocc, 1)
+    eps = np.linspace(-7.0, -3.0, s.nocc)
+    x = synth.make_guess(s, 7, 3)
+    v = np.arange(7) % s.nocc
+    y = {}
+    for variant in (8, 3):
+        with pinned(variant, s, psi, eps, "fp64") as c:
+            assert c.plane_variant(64) == variant
+            y[variant] = (c.apply_sternheimer_operator(v, x), c.apply_hamiltonian(x[:5]))
+    assert rel(y[8][0], y[3][0]) < 1e-14 and rel(y[8][1], y[3][1]) < 1e-14
+    with pinned(8, s, psi, eps) as c:  # H x of a double-float context is FP64 too
+        assert rel(c.apply_hamiltonian(x[:5]), y[3][1]) < 1e-14
+
+
 @pytest.mark.parametrize("n", [24, 45, 64, 96])
 def test_band_edge(n):
     s = probe(n, n // 4)
