@@ -360,7 +360,7 @@ int wdf_train_preconditioner(wdf_ctx *const *ctx, int n, const wdf_train_opts *o
  * by calls on ctx is bracketed by two events recorded on the stream it is launched on.
  * kernel: a class name, optionally with ":64", ":32" or ":48" for the precision, e.g. "plane_vloc:32".
  * Precision suffixes: 64 (FP64), 32 (FP32), 48 (double-float). Classes: zpass_g2r, zpass_r2g, plane_vloc, plane_g2r, plane_prod, plane_accum, gram, gram_sum,
- * lincomb, dot_partial, cg_start, cg_update, cg_direction, cg_scalars, axpby, scale_rows,
+ * lincomb, dot_partial, cg_start, cg_update, cg_scalars, axpby, scale_rows,
  * convert, ext_to_int, int_to_ext, ritz_residual, tpa_table, kinetic, mul_table, check_finite,
  * jac_init, jac_rows, jac_cols, jac_check, jac_sort, split_pairs, scale_elems, gather_shift,
  * sum_chunks, chol_inv, compact, tc_prep, mlp_predict, mlp_grad, mlp_reduce, mlp_adam, mlp_table, mlp_accum, mlp_samples. NULL stops timing. Calling it resets the counters. Errors: WDF_EINVAL. */

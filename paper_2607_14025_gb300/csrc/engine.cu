@@ -378,13 +378,13 @@ static int apply_operator_cg(wdf_ctx *c, cplx<T> *X, cplx<T> *Y, int n, const do
       const size_t need = gram_tc_work_doubles(g, M, n);
       c->gramw.ensure(std::max<size_t>(need, 1) * sizeof(double));
       cap = c->gramw.cap / sizeof(double);
-      launch_gram_tc(g, reinterpret_cast<const float *>(X), n, c->tc_uwh(), c->tc_uwl(), M, w.S.as<double>(), c->gramw.as<double>(),
-                     cap, c->tcerr.as<int>(), c->st);
+      const TcGram sp = launch_gram_tc(g, reinterpret_cast<const float *>(X), n, c->tc_uwh(), c->tc_uwl(), M, w.S.as<double>(),
+                                       c->gramw.as<double>(), cap, c->tcerr.as<int>(), c->st);
       const int kp = tc_rows(M);
       c->tcC.ensure(sizeof(float) * 2 * (size_t)n * kp);
       float *chi = c->tcC.as<float>(), *clo = chi + (size_t)n * kp;
-      launch_lincomb_tc(g, reinterpret_cast<float *>(Y), n, w.S.as<double>(), n, c->lrd.as<double>(), M, chi, clo, c->tc_uth(),
-                        c->tc_utl(), 1.0f, dotpart ? reinterpret_cast<const float *>(X) : nullptr, dotpart, c->tcerr.as<int>(), c->st);
+      launch_lincomb_tc(g, reinterpret_cast<float *>(Y), n, sp, c->lrd.as<double>(), M, chi, clo, c->tc_uth(), c->tc_utl(),
+                        1.0f, dotpart ? reinterpret_cast<const float *>(X) : nullptr, dotpart, c->tcerr.as<int>(), c->st);
       return dotpart ? lincomb_dot_chunks(g) : 0;
     }
   }
@@ -404,20 +404,19 @@ static void cg_solve(wdf_ctx *c, const cplx<T> *b, cplx<T> *x, int n, int maxite
   wdf_ctx::Cg &w = Prec<T>::cg(c);
   const size_t vb = sizeof(cplx<T>) * (size_t)n * g.ld;
   w.r.ensure(vb);
-  w.z.ensure(vb);
   w.p.ensure(vb);
   w.Ap.ensure(vb);
   const int nch = dot_chunks(g);
-  w.part1.ensure(sizeof(double) * (size_t)n * std::max(nch, lincomb_dot_chunks(g)));
+  w.part1.ensure(sizeof(double) * (size_t)n * nch);
+  w.dots.ensure(sizeof(double) * (size_t)n * std::max(nch, lincomb_dot_chunks(g)));
   w.part2.ensure(sizeof(double) * (size_t)n * nch);
-  w.dbl.ensure(sizeof(double) * 4 * (size_t)n);
-  w.ints.ensure(sizeof(int) * (2 * (size_t)n + 1));
+  w.dbl.ensure(sizeof(double) * 3 * (size_t)n);
+  w.ints.ensure(sizeof(int) * (3 * (size_t)n + 2));
   CgState s;
   double *d = w.dbl.as<double>();
   s.rz = d;
   s.rz_new = d + n;
-  s.pap = d + 2 * n;
-  s.rr = d + 3 * n;
+  s.rr = d + 2 * n;
   s.thr = c->thr.as<double>();
   s.shift = c->shift.as<double>();
   s.part1 = w.part1.as<double>();
@@ -425,9 +424,10 @@ static void cg_solve(wdf_ctx *c, const cplx<T> *b, cplx<T> *x, int n, int maxite
   int *ii = w.ints.as<int>();
   s.active = ii;
   s.iters = ii + n;
-  s.nactive = ii + 2 * n;
+  s.arrived = ii + 2 * n;
+  s.nactive = ii + 3 * n;
   s.vidx = c->vidx_dev.as<int>();
-  cplx<T> *r = w.r.as<cplx<T>>(), *z = w.z.as<cplx<T>>(), *p = w.p.as<cplx<T>>(), *Ap = w.Ap.as<cplx<T>>();
+  cplx<T> *r = w.r.as<cplx<T>>(), *p = w.p.as<cplx<T>>(), *Ap = w.Ap.as<cplx<T>>();
   cudaStream_t st = c->st;
   const T *K = c->opt.precond == WDF_PRECOND_TPA ? Prec<T>::kp(c) : nullptr;
   if (c->opt.precond == WDF_PRECOND_LEARNED) {
@@ -446,10 +446,9 @@ static void cg_solve(wdf_ctx *c, const cplx<T> *b, cplx<T> *x, int n, int maxite
 
   WDF_CUDA_TRY(cudaMemsetAsync(x, 0, vb, st));
   WDF_CUDA_TRY(cudaMemcpyAsync(r, b, vb, cudaMemcpyDeviceToDevice, st));
-  WDF_CUDA_TRY(cudaMemsetAsync(ii, 0, sizeof(int) * (2 * (size_t)n + 1), st));
-  (void)z;  // z = K r is not stored: the update and the direction recompute it
-  launch_cg_start<T>(g, r, nullptr, p, K, s, n, nch, st);
-  launch_cg_scalars(s, n, nch, 2, maxiter, st);
+  WDF_CUDA_TRY(cudaMemsetAsync(ii, 0, sizeof(int) * (3 * (size_t)n + 2), st));
+  launch_cg_start<T>(g, r, p, K, s, n, nch, st);
+  launch_cg_scalars(s, n, nch, maxiter, st);
   int nact = 0;
   WDF_CUDA_TRY(cudaMemcpyAsync(&nact, s.nactive, sizeof(int), cudaMemcpyDeviceToHost, st));
   WDF_CUDA_TRY(cudaStreamSynchronize(st));
@@ -514,16 +513,14 @@ static void cg_solve(wdf_ctx *c, const cplx<T> *b, cplx<T> *x, int n, int maxite
     dir.active = s.active;
     dir.beta = s.rz_new;
     // p = K r + beta p (from the second iteration on), A p and the partial sums of <p, A p>
-    int ndot = apply_operator_cg<T>(c, p, Ap, ncur, s.shift, it > 0 ? &dir : nullptr, s.part1);
+    int ndot = apply_operator_cg<T>(c, p, Ap, ncur, s.shift, it > 0 ? &dir : nullptr, w.dots.as<double>());
     if (ndot == 0) {
-      launch_dot_partial<T>(g, p, Ap, ncur, s.part1, nch, st);
+      launch_dot_partial<T>(g, p, Ap, ncur, w.dots.as<double>(), nch, st);
       ndot = nch;
     }
-    launch_cg_scalars(s, ncur, ndot, 0, maxiter, st);
-    launch_cg_update<T>(g, x, r, nullptr, p, Ap, K, s, ncur, nch, st);
-    WDF_CUDA_TRY(cudaMemsetAsync(s.nactive, 0, sizeof(int), st));
-    launch_cg_scalars(s, ncur, nch, 1, maxiter, st);
-    WDF_CUDA_TRY(cudaMemcpyAsync(&nact, s.nactive, sizeof(int), cudaMemcpyDeviceToHost, st));
+    const int which = (it & 1) ^ 1;
+    launch_cg_update<T>(g, x, r, p, Ap, K, s, ncur, w.dots.as<double>(), ndot, maxiter, which, st);
+    WDF_CUDA_TRY(cudaMemcpyAsync(&nact, s.nactive + which, sizeof(int), cudaMemcpyDeviceToHost, st));
     WDF_CUDA_TRY(cudaStreamSynchronize(st));
   }
   if (nset > 0) {

@@ -81,7 +81,7 @@ struct wdf_ctx {
 
   // workspaces (grow-only)
   struct Cg {
-    wdf::DBuf r, z, p, Ap, x, cb, S, part1, part2, part3, dbl, ints;
+    wdf::DBuf r, p, Ap, x, cb, S, dots, part1, part2, part3, dbl, ints;
     wdf::DBuf r2, p2, cd, ci, cidx;  // compacted copies of the active solves' rows and state
   } cg64, cg32, cgdf;
   // learned preconditioner (wdf_set_model): [2 nocc][ld] tables (learned rows, then TPA rows),

@@ -162,13 +162,14 @@ void launch_diff_partial(const Geo &g, const cplx<double> *A, const cplx<float> 
 // ---------------------------------------------------------------------------------------------
 // CG state per solve (device arrays of length n unless noted)
 struct CgState {
-  double *rz, *rz_new, *pap, *rr;       // <r,z>, beta (after the scalar step), <p,Ap>, <r,r>
+  double *rz, *rz_new, *rr;              // <r,z>, beta (after the scalar step), <r,r>
   double *thr;                           // stop a solve once <r,r> <= thr
   double *shift;                         // eps_v of each solve
   double *part1, *part2;                 // partial sums [n * nchunk]
   int *active;                           // 1 while the solve iterates
   int *iters;                            // iterations done
-  int *nactive;                          // [1] count of active solves
+  int *nactive;                          // [2] counts of active solves (alternating between iterations)
+  int *arrived;                          // blocks of each row done with their update (0 between launches)
   int *vidx;                             // preconditioner row of each solve (its orbital for TPA)
   // learned preconditioner only (krow null otherwise): rows [0, nocc) of the table are learned,
   // rows [nocc, 2 nocc) TPA; a solve whose <r,r> falls by less than 19% over 5 iterations (||r||
@@ -185,21 +186,17 @@ struct CgState {
   const int *home = nullptr;
 };
 
-// z = K r (TPA per orbital), p = z, and partials for <r,z>, <r,r>
+// p = K r (TPA per orbital) and partials for <r, K r>, <r, r>
 template <typename T>
-void launch_cg_start(const Geo &g, const cplx<T> *r, cplx<T> *z, cplx<T> *p, const T *kprec, const CgState &s, int n,
-                     int nchunk, cudaStream_t st);
-// alpha = rz / pAp; x += alpha p; r -= alpha Ap; z = K r; partials <r,z>, <r,r> (and, for the
-// learned table, <r, K_TPA r> of the solves still on a learned row)
+void launch_cg_start(const Geo &g, const cplx<T> *r, cplx<T> *p, const T *kprec, const CgState &s, int n, int nchunk, cudaStream_t st);
+// after launch_cg_start: rz, rr, the active solves and their count nactive[0]
+void launch_cg_scalars(const CgState &s, int n, int nchunk, int maxiter, cudaStream_t st);
+// alpha = rz / sum of the row's ndot partials of <p, A p>; x += alpha p; r -= alpha A p; new rz, beta and
+// rr, the stopping test (rr <= thr), iteration counts and, for the learned table, the stall rule; the solves
+// still active are counted in nactive[which], nactive[1 - which] is zeroed
 template <typename T>
-void launch_cg_update(const Geo &g, cplx<T> *x, cplx<T> *r, cplx<T> *z, const cplx<T> *p, const cplx<T> *Ap,
-                      const T *kprec, const CgState &s, int n, int nchunk, cudaStream_t st);
-// p = z + beta p for active solves
-template <typename T>
-void launch_cg_direction(const Geo &g, cplx<T> *p, const cplx<T> *z, const CgState &s, int n, cudaStream_t st);
-// reduce partials: which = 0 -> pap from part1; which = 1 -> new <r,z> from part1, rr from part2,
-// then the stopping test rr <= thr, beta and iteration counting; which = 2: rz, rr at start
-void launch_cg_scalars(const CgState &s, int n, int nchunk, int which, int maxiter, cudaStream_t st);
+void launch_cg_update(const Geo &g, cplx<T> *x, cplx<T> *r, const cplx<T> *p, const cplx<T> *Ap, const T *kprec, const CgState &s, int n,
+                      const double *dots, int ndot, int maxiter, int which, cudaStream_t st);
 
 // elementwise helpers
 template <typename T> void launch_axpby(const Geo &g, cplx<T> *y, const cplx<T> *x, int n, double a, double b, cudaStream_t st);
@@ -260,11 +257,17 @@ void launch_tc_prep_u(const Geo &g, const float2 *U, int na, float *uwh, float *
 // most rows of U ([beta; psi]) the tensor-core projections take (memory of the hi/lo copies only)
 constexpr int kTcMaxRows = 4096;
 size_t gram_tc_work_doubles(const Geo &g, int na, int nb);
-// out[j][s] (ldo = nb) = sum_e w_e Re(conj(U_j) X_s) for j < na, s < nb
-void launch_gram_tc(const Geo &g, const float *X, int nb, const float *uwh, const float *uwl, int na, double *out, double *work,
-                    size_t work_cap, int *err, cudaStream_t st);
+// S[j][s] (row stride nb) = sum_e w_e Re(conj(U_j) X_s) for j < na, s < nb, as the sum of nsplit partial
+// matrices `stride` apart: in out when nsplit is 1, else in work
+struct TcGram {
+  const double *S;
+  int nsplit;
+  size_t stride;
+};
+TcGram launch_gram_tc(const Geo &g, const float *X, int nb, const float *uwh, const float *uwl, int na, double *out, double *work,
+                      size_t work_cap, int *err, cudaStream_t st);
 // Y_s = c0 Y_s + sum_j U_j S[j][s] d_j, partial <P_s, Y_s> per 128-element tile when part != null
-void launch_lincomb_tc(const Geo &g, float *Y, int ny, const double *S, int ldc, const double *d, int na, float *chi, float *clo,
+void launch_lincomb_tc(const Geo &g, float *Y, int ny, const TcGram &S, const double *d, int na, float *chi, float *clo,
                        const float *uth, const float *utl, float c0, const float *P, double *part, int *err, cudaStream_t st);
 
 // double-float projections on the tensor cores by exact integer digits (oz_gemm.cu); on with the

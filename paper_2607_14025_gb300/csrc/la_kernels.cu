@@ -746,8 +746,7 @@ void launch_diff_partial(const Geo &g, const cplx<double> *A, const cplx<float> 
 // conjugate gradients
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_cg_start(Geo g, const cplx<T> *__restrict__ r, cplx<T> *z,
-                                                 cplx<T> *__restrict__ p, const T *__restrict__ kprec, CgState s, int nchunk) {
+__global__ void __launch_bounds__(256) k_cg_start(Geo g, const cplx<T> *__restrict__ r, cplx<T> *__restrict__ p, const T *__restrict__ kprec, CgState s, int nchunk) {
   const int i = blockIdx.x, c = blockIdx.y;
   const int e0 = c * DCHUNK, e1 = min(g.nint, e0 + DCHUNK);
   const size_t o = (size_t)i * g.ld;
@@ -758,7 +757,6 @@ __global__ void __launch_bounds__(256) k_cg_start(Geo g, const cplx<T> *__restri
     const cplx<T> rv = r[o + e];
     const T k = K ? K[e] : (T)1;
     const cplx<T> zv = mkc<T>(k * rv.x, k * rv.y);
-    if (z) z[o + e] = zv;
     p[o + e] = zv;
     const A w = e < g.len0 ? (A)1 : (A)2;
     vrz += w * dre_acc<T>(rv, zv);
@@ -773,45 +771,128 @@ __global__ void __launch_bounds__(256) k_cg_start(Geo g, const cplx<T> *__restri
 }
 
 template <typename T>
-void launch_cg_start(const Geo &g, const cplx<T> *r, cplx<T> *z, cplx<T> *p, const T *kprec, const CgState &s, int n, int nchunk,
+void launch_cg_start(const Geo &g, const cplx<T> *r, cplx<T> *p, const T *kprec, const CgState &s, int n, int nchunk,
                      cudaStream_t st) {
   if (n <= 0) return;
-  launch("cg_start", bits_of<T>(), k_cg_start<T>, dim3(dim3(n, nchunk)), dim3(256), 0, st, g, r, z, p, kprec, s, nchunk);
+  launch("cg_start", bits_of<T>(), k_cg_start<T>, dim3(dim3(n, nchunk)), dim3(256), 0, st, g, r, p, kprec, s, nchunk);
   WDF_CUDA_TRY(cudaGetLastError());
 }
 
+// block_sum with the result in every thread
+static __device__ double block_sum_all(double v) {
+  __shared__ double bc;
+  v = block_sum(v);
+  if (threadIdx.x == 0) bc = v;
+  __syncthreads();
+  return bc;
+}
+
+// One CG update per launch: alpha from the partial sums of <p, A p>, x += alpha p, r -= alpha A p, the
+// partial sums of <r, K r> and <r, r>, and, in the last block of each solve to finish, the scalar step
+// (beta, the stopping test, the stall rule of the learned preconditioner). With the scalar steps and the
+// counter's reset as launches of their own (two k_cg_scalars, a memset) small systems spent 5 of 12
+// stream operations an iteration on them. At size the kernel is bound by HBM (x, r, p, A p read, x, r
+// written): 16-byte accesses, UB of each array in flight per thread, the first ones before the sum that
+// gives alpha, and longer chunks when the rows alone fill the SMs. Row i has the
+// blocks (i, 0 .. nchunk - 1); every sum runs in a fixed order, so it does not matter which of them
+// finishes last.
+template <typename T> struct UpdVec;  // 16 bytes of a vector
+template <> struct UpdVec<float> {
+  typedef float4 V;
+  typedef float2 K;
+  static constexpr int E = 2;
+};
+template <> struct UpdVec<double> {
+  typedef double2 V;
+  typedef double K;
+  static constexpr int E = 1;
+};
+__device__ __forceinline__ void upd_elems(float4 v, float2 (&e)[2]) {
+  e[0] = make_float2(v.x, v.y);
+  e[1] = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void upd_elems(double2 v, double2 (&e)[1]) { e[0] = v; }
+__device__ __forceinline__ float4 upd_vec(const float2 (&e)[2]) { return make_float4(e[0].x, e[0].y, e[1].x, e[1].y); }
+__device__ __forceinline__ double2 upd_vec(const double2 (&e)[1]) { return e[0]; }
+__device__ __forceinline__ void upd_k(float2 v, float (&k)[2]) {
+  k[0] = v.x;
+  k[1] = v.y;
+}
+__device__ __forceinline__ void upd_k(double v, double (&k)[1]) { k[0] = v; }
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_cg_update(Geo g, cplx<T> *__restrict__ x, cplx<T> *__restrict__ r, cplx<T> *z,
-                                                  const cplx<T> *__restrict__ p, const cplx<T> *__restrict__ Ap,
-                                                  const T *__restrict__ kprec, CgState s, int nchunk) {
-  const int i = blockIdx.x, c = blockIdx.y;
+__global__ void __launch_bounds__(256) k_cg_update(Geo g, cplx<T> *__restrict__ x, cplx<T> *__restrict__ r, const cplx<T> *__restrict__ p,
+                                                  const cplx<T> *__restrict__ Ap, const T *__restrict__ kprec, CgState s, int nchunk,
+                                                  int chunk, const double *__restrict__ dots, int ndot, int maxiter, int which) {
   typedef PartAcc<T> A;
-  A vrz = 0, vrr = 0, vr3 = 0;
+  typedef typename UpdVec<T>::V V;
+  typedef typename UpdVec<T>::K KV;
+  constexpr int E = UpdVec<T>::E, UB = 2, STEP = 256 * E * UB;
+  const int i = blockIdx.x, c = blockIdx.y;
+  __shared__ int last;
+  if (i == 0 && c == 0 && threadIdx.x == 0) s.nactive[which ^ 1] = 0;  // the next launch's count
+  if (!s.active[i]) return;
   // learned table: also <r, K_TPA r> while the solve is on its learned row (for a restart)
   const bool fb = s.krow && s.krow[i] < s.nocc;
-  if (s.active[i]) {
-    const int e0 = c * DCHUNK, e1 = min(g.nint, e0 + DCHUNK);
-    const size_t o = (size_t)i * g.ld, ox = (size_t)(s.home ? s.home[i] : i) * g.ld;
-    const T *K = kprec ? kprec + (size_t)s.vidx[i] * g.ld : nullptr;
-    const T *K3 = fb ? kprec + (size_t)(s.vorig[i] + s.nocc) * g.ld : nullptr;
-    const T al = (T)(s.rz[i] / s.pap[i]);
-    for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-      const cplx<T> pv = p[o + e], av = Ap[o + e];
-      cplx<T> xv = x[ox + e], rv = r[o + e];
-      xv.x += al * pv.x;
-      xv.y += al * pv.y;
-      rv.x -= al * av.x;
-      rv.y -= al * av.y;
-      x[ox + e] = xv;
-      r[o + e] = rv;
-      const T k = K ? K[e] : (T)1;
-      const cplx<T> zv = mkc<T>(k * rv.x, k * rv.y);
-      if (z) z[o + e] = zv;  // z = K r is recomputed where needed when not stored
-      const A w = e < g.len0 ? (A)1 : (A)2;
-      const A rr = dre_acc<T>(rv, rv);
-      vrz += w * dre_acc<T>(rv, zv);
-      vrr += w * rr;
-      if (K3) vr3 += w * (A)K3[e] * rr;
+  const int e0 = c * chunk, e1 = min(g.nint, e0 + chunk);
+  const size_t o = (size_t)i * g.ld, ox = (size_t)(s.home ? s.home[i] : i) * g.ld;
+  const T *K = kprec ? kprec + (size_t)s.vidx[i] * g.ld : nullptr;
+  const T *K3 = fb ? kprec + (size_t)(s.vorig[i] + s.nocc) * g.ld : nullptr;
+  V pv[UB], av[UB], xv[UB], rv[UB];
+  // rows are padded to a multiple of 32 elements, so a vector that starts inside a row ends inside it
+  auto load = [&](int e) {
+#pragma unroll
+    for (int u = 0; u < UB; ++u) {
+      const int eu = e + u * 256 * E;
+      if (eu < e1) {
+        av[u] = *reinterpret_cast<const V *>(Ap + o + eu);
+        rv[u] = *reinterpret_cast<const V *>(r + o + eu);
+        pv[u] = *reinterpret_cast<const V *>(p + o + eu);
+        xv[u] = *reinterpret_cast<const V *>(x + ox + eu);
+      }
+    }
+  };
+  int e = e0 + (int)threadIdx.x * E;
+  load(e);
+  double pap = 0.0;
+  for (int k = threadIdx.x; k < ndot; k += blockDim.x) pap += dots[(size_t)i * ndot + k];
+  pap = block_sum_all(pap);
+  if (!(pap > 0.0)) {  // breakdown: keep the current iterate (every block of the row sees the same sum)
+    if (c == 0 && threadIdx.x == 0) s.active[i] = 0;
+    return;
+  }
+  const T al = (T)(s.rz[i] / pap);
+  A vrz = 0, vrr = 0, vr3 = 0;
+  for (; e < e1; e += STEP, load(e)) {
+#pragma unroll
+    for (int u = 0; u < UB; ++u) {
+      const int eu = e + u * 256 * E;
+      if (eu >= e1) break;
+      cplx<T> pe[E], ae[E], xe[E], re[E];
+      T ke[E], k3[E];
+      upd_elems(pv[u], pe);
+      upd_elems(av[u], ae);
+      upd_elems(xv[u], xe);
+      upd_elems(rv[u], re);
+      if (K) upd_k(*reinterpret_cast<const KV *>(K + eu), ke);
+      if (K3) upd_k(*reinterpret_cast<const KV *>(K3 + eu), k3);
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        xe[q].x += al * pe[q].x;
+        xe[q].y += al * pe[q].y;
+        re[q].x -= al * ae[q].x;
+        re[q].y -= al * ae[q].y;
+        if (eu + q >= e1) continue;  // an element of row padding (zero, and stays zero)
+        const T k = K ? ke[q] : (T)1;
+        const cplx<T> zv = mkc<T>(k * re[q].x, k * re[q].y);  // z = K r, recomputed where it is needed
+        const A w = eu + q < g.len0 ? (A)1 : (A)2;
+        const A rr = dre_acc<T>(re[q], re[q]);
+        vrz += w * dre_acc<T>(re[q], zv);
+        vrr += w * rr;
+        if (K3) vr3 += w * (A)k3[q] * rr;
+      }
+      *reinterpret_cast<V *>(x + ox + eu) = upd_vec(xe);
+      *reinterpret_cast<V *>(r + o + eu) = upd_vec(re);
     }
   }
   const double brz = block_sum((double)vrz);
@@ -821,89 +902,76 @@ __global__ void __launch_bounds__(256) k_cg_update(Geo g, cplx<T> *__restrict__ 
     s.part1[(size_t)i * nchunk + c] = brz;
     s.part2[(size_t)i * nchunk + c] = brr;
     if (fb) s.part3[(size_t)i * nchunk + c] = br3;
+    __threadfence();
+    last = atomicAdd(&s.arrived[i], 1) == nchunk - 1;
   }
-}
-
-template <typename T>
-void launch_cg_update(const Geo &g, cplx<T> *x, cplx<T> *r, cplx<T> *z, const cplx<T> *p, const cplx<T> *Ap, const T *kprec,
-                      const CgState &s, int n, int nchunk, cudaStream_t st) {
-  if (n <= 0) return;
-  launch("cg_update", bits_of<T>(), k_cg_update<T>, dim3(dim3(n, nchunk)), dim3(256), 0, st, g, x, r, z, p, Ap, kprec, s, nchunk);
-  WDF_CUDA_TRY(cudaGetLastError());
-}
-
-template <typename T>
-__global__ void k_cg_direction(Geo g, cplx<T> *__restrict__ p, const cplx<T> *__restrict__ z, CgState s, int n) {
-  const int i = blockIdx.x;
-  if (!s.active[i]) return;
-  const T be = (T)s.rz_new[i];  // holds beta after the scalar step
-  const size_t o = (size_t)i * g.ld;
-  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < g.nint; e += gridDim.y * blockDim.x) {
-    const cplx<T> zv = z[o + e], pv = p[o + e];
-    p[o + e] = mkc<T>(zv.x + be * pv.x, zv.y + be * pv.y);
-  }
-}
-
-template <typename T>
-void launch_cg_direction(const Geo &g, cplx<T> *p, const cplx<T> *z, const CgState &s, int n, cudaStream_t st) {
-  if (n <= 0) return;
-  const int by = std::min(64, (g.nint + 255) / 256);
-  launch("cg_direction", bits_of<T>(), k_cg_direction<T>, dim3(dim3(n, by)), dim3(256), 0, st, g, p, z, s, n);
-  WDF_CUDA_TRY(cudaGetLastError());
-}
-
-__global__ void k_cg_scalars(CgState s, int n, int nchunk, int which, int maxiter) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  __syncthreads();
+  if (!last || threadIdx.x != 0) return;
+  __threadfence();
+  s.arrived[i] = 0;
+  const volatile double *q1 = s.part1 + (size_t)i * nchunk, *q2 = s.part2 + (size_t)i * nchunk, *q3 = s.part3 + (size_t)i * nchunk;
   double a = 0.0, b = 0.0;
-  for (int c = 0; c < nchunk; ++c) a += s.part1[(size_t)i * nchunk + c];
-  if (which != 0)
-    for (int c = 0; c < nchunk; ++c) b += s.part2[(size_t)i * nchunk + c];
-  if (which == 0) {
-    s.pap[i] = a;
-    if (s.active[i] && !(a > 0.0)) s.active[i] = 0;  // breakdown: keep the current iterate
-    return;
-  }
-  if (which == 2) {  // start: r = b - A x0, z = K r
-    s.rz[i] = a;
-    s.rr[i] = b;
-    const int act = (b > s.thr[i]) && (b > 0.0) && (s.iters[i] < maxiter);
-    s.active[i] = act;
-    if (act) atomicAdd(s.nactive, 1);
-    if (s.krow) {
-      s.rr_ref[i] = b;
-      s.it_ref[i] = s.iters[i];
-    }
-    return;
-  }
-  if (!s.active[i]) return;
-  s.iters[i] += 1;
+  for (int k = 0; k < nchunk; ++k) a += q1[k];
+  for (int k = 0; k < nchunk; ++k) b += q2[k];
+  const int it = s.iters[i] + 1;
+  s.iters[i] = it;
   s.rr[i] = b;
   const double beta = a / s.rz[i];
   s.rz[i] = a;
   s.rz_new[i] = beta;
-  if (b <= s.thr[i] || s.iters[i] >= maxiter || !(b == b)) {
+  if (b <= s.thr[i] || it >= maxiter || !(b == b)) {
     s.active[i] = 0;
     return;
   }
-  atomicAdd(s.nactive, 1);
-  if (s.krow && s.krow[i] < s.nocc && s.iters[i] - s.it_ref[i] >= 5) {
+  atomicAdd(&s.nactive[which], 1);
+  if (s.krow && s.krow[i] < s.nocc && it - s.it_ref[i] >= 5) {
     if (b > 0.81 * s.rr_ref[i]) {  // stalled on the learned row: TPA from the current iterate
       double c3 = 0.0;
-      for (int c = 0; c < nchunk; ++c) c3 += s.part3[(size_t)i * nchunk + c];
+      for (int k = 0; k < nchunk; ++k) c3 += q3[k];
       s.krow[i] = s.vorig[i] + s.nocc;
       s.rz[i] = c3;
       s.rz_new[i] = 0.0;  // beta = 0: p = K_TPA r
       atomicAdd(s.nfb, 1);
     }
     s.rr_ref[i] = b;
+    s.it_ref[i] = it;
+  }
+}
+
+template <typename T>
+void launch_cg_update(const Geo &g, cplx<T> *x, cplx<T> *r, const cplx<T> *p, const cplx<T> *Ap, const T *kprec, const CgState &s, int n,
+                      const double *dots, int ndot, int maxiter, int which, cudaStream_t st) {
+  if (n <= 0) return;
+  // DCHUNK elements a block; four times as many once that still leaves four blocks for each of the
+  // 152 SMs twice over, so that a block's start and sums weigh less
+  const int chunk = (long)n * ((g.nint + 4 * DCHUNK - 1) / (4 * DCHUNK)) >= 8 * 152 ? 4 * DCHUNK : DCHUNK;
+  const int nchunk = (g.nint + chunk - 1) / chunk;
+  launch("cg_update", bits_of<T>(), k_cg_update<T>, dim3(n, nchunk), dim3(256), 0, st, g, x, r, p, Ap, kprec, s, nchunk, chunk, dots, ndot,
+         maxiter, which);
+  WDF_CUDA_TRY(cudaGetLastError());
+}
+
+// after k_cg_start: <r, K r>, <r, r>, and which solves iterate
+__global__ void k_cg_scalars(CgState s, int n, int nchunk, int maxiter) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double a = 0.0, b = 0.0;
+  for (int c = 0; c < nchunk; ++c) a += s.part1[(size_t)i * nchunk + c];
+  for (int c = 0; c < nchunk; ++c) b += s.part2[(size_t)i * nchunk + c];
+  s.rz[i] = a;
+  s.rr[i] = b;
+  const int act = (b > s.thr[i]) && (b > 0.0) && (s.iters[i] < maxiter);
+  s.active[i] = act;
+  if (act) atomicAdd(s.nactive, 1);
+  if (s.krow) {
+    s.rr_ref[i] = b;
     s.it_ref[i] = s.iters[i];
   }
 }
 
-void launch_cg_scalars(const CgState &s, int n, int nchunk, int which, int maxiter, cudaStream_t st) {
+void launch_cg_scalars(const CgState &s, int n, int nchunk, int maxiter, cudaStream_t st) {
   if (n <= 0) return;
-  launch("cg_scalars", 0, k_cg_scalars, dim3((n + 127) / 128), dim3(128), 0, st, s, n, nchunk, which, maxiter);
+  launch("cg_scalars", 0, k_cg_scalars, dim3((n + 127) / 128), dim3(128), 0, st, s, n, nchunk, maxiter);
   WDF_CUDA_TRY(cudaGetLastError());
 }
 
@@ -1602,11 +1670,10 @@ void jacobi_eigh(double *Ain, double *Vout, double *w, int n, double *work, int 
   template void launch_lincomb<T>(const Geo &, cplx<T> *, int, const cplx<T> *, int, const double *, int, const double *, \
                                   double, cudaStream_t);                                                              \
   template void launch_dot_partial<T>(const Geo &, const cplx<T> *, const cplx<T> *, int, double *, int, cudaStream_t); \
-  template void launch_cg_start<T>(const Geo &, const cplx<T> *, cplx<T> *, cplx<T> *, const T *, const CgState &, int,  \
-                                   int, cudaStream_t);                                                                \
-  template void launch_cg_update<T>(const Geo &, cplx<T> *, cplx<T> *, cplx<T> *, const cplx<T> *, const cplx<T> *,     \
-                                    const T *, const CgState &, int, int, cudaStream_t);                             \
-  template void launch_cg_direction<T>(const Geo &, cplx<T> *, const cplx<T> *, const CgState &, int, cudaStream_t);   \
+  template void launch_cg_start<T>(const Geo &, const cplx<T> *, cplx<T> *, const T *, const CgState &, int, int,       \
+                                   cudaStream_t);                                                                     \
+  template void launch_cg_update<T>(const Geo &, cplx<T> *, cplx<T> *, const cplx<T> *, const cplx<T> *, const T *,     \
+                                    const CgState &, int, const double *, int, int, int, cudaStream_t);              \
   template bool launch_lincomb_dot<T>(const Geo &, cplx<T> *, int, const cplx<T> *, int, const double *, int, const double *, \
                                       double, const cplx<T> *, double *, cudaStream_t);                              \
   template void launch_axpby<T>(const Geo &, cplx<T> *, const cplx<T> *, int, double, double, cudaStream_t);          \

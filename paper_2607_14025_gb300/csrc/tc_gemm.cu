@@ -217,26 +217,29 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram_tc(const __grid_consta
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
-__global__ void k_tc_sum_splits(const double *__restrict__ work, int nsplit, size_t stride, double *__restrict__ out, int na, int nb,
-                                int ldo) {
-  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (t >= (size_t)na * nb) return;
-  const int j = (int)(t / nb), s = (int)(t % nb);
-  double a = 0.0;
-  for (int k = 0; k < nsplit; ++k) a += work[k * stride + (size_t)j * ldo + s];
-  out[(size_t)j * ldo + s] = a;
-}
-
-// Cd[s][j] = S[j][s] d_j (j < na, else 0), hi and lo parts, through a 32 x 32 shared tile
-__global__ void k_tc_coef(const double *__restrict__ S, int ldc, const double *__restrict__ d, int na, int nb, int kp,
-                          float *__restrict__ hi, float *__restrict__ lo) {
+// Cd[s][j] = d_j sum over the splits of S[j][s] (j < na, else 0), hi and lo parts, through a 32 x 32
+// shared tile: the K splits of the Gram are added here, where they are read anyway
+__global__ void k_tc_coef(const double *__restrict__ S, int nsplit, size_t stride, int ldc, const double *__restrict__ d, int na, int nb,
+                          int kp, float *__restrict__ hi, float *__restrict__ lo) {
   __shared__ float tile[32][33];
   const int j0 = blockIdx.y * 32, s0 = blockIdx.x * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int j = j0 + r, s = s0 + threadIdx.x;
-    float v = 0.f;
-    if (j < na && s < nb) v = (float)(S[(size_t)j * ldc + s] * (d ? d[j] : 1.0));
-    tile[r][threadIdx.x] = v;
+  {  // four rows of S per thread (blockDim.y = 8), their splits' loads in flight together
+    const int s = s0 + threadIdx.x;
+    const double *q = S + (size_t)(j0 + threadIdx.y) * ldc + s;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    bool on[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) on[u] = s < nb && j0 + (int)threadIdx.y + 8 * u < na;
+#pragma unroll 4
+    for (int k = 0; k < nsplit; ++k)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (on[u]) a[u] += q[k * stride + (size_t)(8 * u) * ldc];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = j0 + threadIdx.y + 8 * u;
+      tile[threadIdx.y + 8 * u][threadIdx.x] = on[u] ? (float)(a[u] * (d ? d[j] : 1.0)) : 0.f;
+    }
   }
   __syncthreads();
   for (int r = threadIdx.y; r < 32; r += blockDim.y) {
@@ -480,23 +483,25 @@ void launch_tc_prep_u(const Geo &g, const float2 *U, int na, float *uwh, float *
 }
 
 // K splits of the Gram: one CTA per SM (shared memory), so the launch runs in waves of nsm CTAs;
-// choose the split count (at most nch / 16, so that each CTA keeps a pipeline of >= 16 chunks)
-// that minimises waves x (chunks per CTA + 12), the 12 standing for a CTA's partial-sum write
-// (128 x 192 doubles, about the bytes of two dozen 16-value X chunks, written without waiting),
-// the smaller count on ties (fewer partial sums to add)
-static int gram_tc_splits(int nch, int tiles) {
+// choose the split count (at most nch / 4, so that each CTA fills its four stages) that minimises
+// waves x (chunks per CTA + 12) + sums, the 12 standing for a CTA's partial-sum write (128 x 192
+// doubles, about the bytes of two dozen 16-value X chunks, written without waiting) and the sums for
+// the partial matrices that k_tc_coef reads (8 na nb bytes each at about 4 TB/s, a chunk taking about a
+// microsecond); the smaller count on ties. Small systems are latency-bound: 18 rows x 60 vectors of
+// 710 waves 13.3 us in 5 CTAs of 18 chunks (the bound was nch / 16), 8.0 us in 22 of 4.
+static int gram_tc_splits(int nch, int tiles, int na, int nb) {
   static int nsm = 0;
   if (nsm == 0) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
       nsm = 152;
   }
-  const int smax = std::max(1, std::min(nch / 16, 4 * ((nsm + tiles - 1) / tiles)));
-  long best = -1;
+  const int smax = std::max(1, std::min(nch / 4, 4 * ((nsm + tiles - 1) / tiles)));
+  double best = -1;
   int bs = 1;
   for (int sp = 1; sp <= smax; ++sp) {
     const long waves = ((long)tiles * sp + nsm - 1) / nsm, per = (nch + sp - 1) / sp;
-    const long cost = waves * (per + 12);
+    const double cost = (double)(waves * (per + 12)) + (sp > 1 ? sp * ((double)na * nb / 500000.0) : 0.0);
     if (best < 0 || cost < best) {
       best = cost;
       bs = sp;
@@ -508,7 +513,7 @@ static int gram_tc_splits(int nch, int tiles) {
 size_t gram_tc_work_doubles(const Geo &g, int na, int nb) {
   const int nch = (2 * g.nint + kGramK - 1) / kGramK;
   const int tiles = ((nb + TM - 1) / TM) * ((na + kGramRows - 1) / kGramRows);
-  const int nsplit = gram_tc_splits(nch, tiles);
+  const int nsplit = gram_tc_splits(nch, tiles, na, nb);
   return nsplit > 1 ? (size_t)nsplit * na * nb : 0;
 }
 
@@ -527,15 +532,15 @@ static CUtensorMap rows_map(const float *base, int kf, int rows, int ldf, int bo
   return m;
 }
 
-void launch_gram_tc(const Geo &g, const float *X, int nb, const float *uwh, const float *uwl, int na, double *out, double *work,
+TcGram launch_gram_tc(const Geo &g, const float *X, int nb, const float *uwh, const float *uwl, int na, double *out, double *work,
                     size_t work_cap, int *err, cudaStream_t st) {
-  if (nb <= 0 || na <= 0) return;
+  if (nb <= 0 || na <= 0) return {out, 1, 0};
   const int nmc = (na + kGramRows - 1) / kGramRows;
   const int nbox = tc_rows((na + nmc - 1) / nmc);  // even chunks of U rows
   const int kf = 2 * g.nint, ldf = 2 * g.ld;
   const int nch = (kf + kGramK - 1) / kGramK;
   const int tiles = (nb + TM - 1) / TM;
-  int nsplit = gram_tc_splits(nch, tiles * nmc);
+  int nsplit = gram_tc_splits(nch, tiles * nmc, na, nb);
   if ((size_t)nsplit * na * nb > work_cap) nsplit = 1;
   const int per = (nch + nsplit - 1) / nsplit;
   nsplit = (nch + per - 1) / per;
@@ -545,18 +550,15 @@ void launch_gram_tc(const Geo &g, const float *X, int nb, const float *uwh, cons
   launch("gram", 32, k_gram_tc, dim3(tiles, nsplit, nmc), dim3(kGramThreads), gram_tc_smem(nbox), st, mX, mUh, mUl, g, nb, na, nbox, dst,
          nb, per, stride, err);
   WDF_CUDA_TRY(cudaGetLastError());
-  if (nsplit > 1) {
-    launch("gram_sum", 0, k_tc_sum_splits, dim3((unsigned)(((size_t)na * nb + 255) / 256)), dim3(256), 0, st, (const double *)work,
-           nsplit, stride, out, na, nb, nb);
-    WDF_CUDA_TRY(cudaGetLastError());
-  }
+  return {dst, nsplit, stride};
 }
 
-void launch_lincomb_tc(const Geo &g, float *Y, int ny, const double *S, int ldc, const double *d, int na, float *chi, float *clo,
+void launch_lincomb_tc(const Geo &g, float *Y, int ny, const TcGram &S, const double *d, int na, float *chi, float *clo,
                        const float *uth, const float *utl, float c0, const float *P, double *part, int *err, cudaStream_t st) {
   if (ny <= 0) return;
   const int kp = tc_rows(na);
-  launch("lincomb", 32, k_tc_coef, dim3((ny + 31) / 32, (kp + 31) / 32), dim3(32, 8), 0, st, S, ldc, d, na, ny, kp, chi, clo);
+  launch("lincomb", 32, k_tc_coef, dim3((ny + 31) / 32, (kp + 31) / 32), dim3(32, 8), 0, st, S.S, S.nsplit, S.stride, ny, d, na, ny, kp,
+         chi, clo);
   WDF_CUDA_TRY(cudaGetLastError());
   const int ntile = (2 * g.nint + kLinTN - 1) / kLinTN;
   const CUtensorMap mCh = rows_map(chi, kp, ny, kp, TM), mCl = rows_map(clo, kp, ny, kp, TM);
