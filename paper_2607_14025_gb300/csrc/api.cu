@@ -455,6 +455,9 @@ void wdf_destroy(wdf_ctx *c) {
                   &c->ozXe,      &c->ozC,       &c->ozCe};
   for (DBuf *b : bufs) b->release();
   for (cudaEvent_t e : c->prof.ev) (void)cudaEventDestroy(e);
+  for (cudaEvent_t e : c->cg_ev)
+    if (e) (void)cudaEventDestroy(e);
+  if (c->cg_count) (void)cudaFreeHost(c->cg_count);
   for (wdf_ctx::Cg *w : {&c->cg64, &c->cg32, &c->cgdf}) {
     DBuf *cb[] = {&w->r,     &w->dots,  &w->p,     &w->Ap, &w->x,  &w->cb, &w->S,  &w->part1,
                   &w->part2, &w->part3, &w->dbl, &w->ints, &w->r2, &w->p2, &w->cd, &w->ci, &w->cidx};

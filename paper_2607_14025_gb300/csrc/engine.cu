@@ -505,8 +505,28 @@ static void cg_solve(wdf_ctx *c, const cplx<T> *b, cplx<T> *x, int n, int maxite
   };
   PDir<T> dir;
   dir.K = K;
+  // The count of an iteration reaches the host while the next one runs: short iterations are launched
+  // one ahead of it, so that the GPU does not idle for the round trip (about 40 us, half of an
+  // iteration on a 30^3 system). A solve that has stopped ignores the iteration launched too many, and
+  // a compaction waits for the exact count. Iterations whose column buffer exceeds kAheadBytes (about
+  // 120 us of kernels) read their own count first: a compaction that comes an iteration late would
+  // cost them more than the round trip.
+  constexpr size_t kAheadBytes = (size_t)16 << 20;
+  bool pending = false;  // the previous iteration's count has not been read
+  auto read_count = [&](int w) {
+    WDF_CUDA_TRY(cudaEventSynchronize(c->cg_ev[w]));
+    nact = *(volatile int *)(c->cg_count + w);
+  };
   for (int it = 0; it < maxiter && nact > 0; ++it) {
-    if (compaction && nact <= ncur - std::max(8, ncur / 8)) compact();
+    const int which = (it & 1) ^ 1;
+    if (compaction && nact <= ncur - std::max(8, ncur / 8)) {
+      if (pending) {
+        read_count(which ^ 1);
+        pending = false;
+        if (nact <= 0) break;
+      }
+      compact();
+    }
     dir.p = p;
     dir.r = r;
     dir.vidx = s.vidx;
@@ -518,10 +538,15 @@ static void cg_solve(wdf_ctx *c, const cplx<T> *b, cplx<T> *x, int n, int maxite
       launch_dot_partial<T>(g, p, Ap, ncur, w.dots.as<double>(), nch, st);
       ndot = nch;
     }
-    const int which = (it & 1) ^ 1;
     launch_cg_update<T>(g, x, r, p, Ap, K, s, ncur, w.dots.as<double>(), ndot, maxiter, which, st);
-    WDF_CUDA_TRY(cudaMemcpyAsync(&nact, s.nactive + which, sizeof(int), cudaMemcpyDeviceToHost, st));
-    WDF_CUDA_TRY(cudaStreamSynchronize(st));
+    WDF_CUDA_TRY(cudaMemcpyAsync(c->cg_count + which, s.nactive + which, sizeof(int), cudaMemcpyDeviceToHost, st));
+    WDF_CUDA_TRY(cudaEventRecord(c->cg_ev[which], st));
+    if (pending) read_count(which ^ 1);
+    pending = true;
+    if (sizeof(cplx<T>) * (size_t)((ncur + 1) / 2) * g.n3 * g.ldcb > kAheadBytes) {
+      read_count(which);
+      pending = false;
+    }
   }
   if (nset > 0) {
     launch("compact", 0, k_scatter_home, dim3((ncur + 127) / 128), dim3(128), 0, st, cur, ncur, ii + n,
@@ -1265,6 +1290,10 @@ template <typename T> static void autotune_vloc(wdf_ctx *c, FftCtx<T> &f, const 
 void finish_setup(wdf_ctx *c) {
   const Geo &g = c->geo;
   cudaStream_t st = c->st;
+  if (!c->cg_count) {
+    WDF_CUDA_TRY(cudaMallocHost(&c->cg_count, 2 * sizeof(int)));
+    for (cudaEvent_t &e : c->cg_ev) WDF_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  }
   const int nocc = c->nocc, M = c->nproj + nocc;
   double emin = c->eps[0], emax = c->eps[0];
   for (double e : c->eps) {

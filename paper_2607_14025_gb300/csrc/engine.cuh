@@ -79,6 +79,10 @@ struct wdf_ctx {
   wdf::DBuf vlocdf, Udf, psirdf;  // double-float copies (WDF_MIXED_DF)
   wdf::DBuf eps_dev;         // [nocc]
 
+  // counts of the active solves on their way to the host: pinned, one per iteration in flight
+  int *cg_count = nullptr;
+  cudaEvent_t cg_ev[2] = {nullptr, nullptr};
+
   // workspaces (grow-only)
   struct Cg {
     wdf::DBuf r, p, Ap, x, cb, S, dots, part1, part2, part3, dbl, ints;
