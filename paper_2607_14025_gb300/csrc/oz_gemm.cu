@@ -315,15 +315,28 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(const __grid_constant
 // ---------------------------------------------------------------------------------------------
 // slicing
 
-// balanced base-128 digits of an integer |I| <= 2^(7T): d[T-1] .. d[1] in [-64, 63], d[0] the rest
+// balanced base-128 digits of an integer |I| <= 2^(7T), T = 7: d[6] .. d[1] in [-64, 63], d[0] the rest.
+// The four lowest digits come from the low 28 bits and a carry into the rest, so everything after the
+// split is 32-bit; a digit becomes a float by adding it to the bits of 1.5 x 2^23 (the integer
+// conversions run at an eighth of the rate).
+__device__ __forceinline__ float oz_small_float(int m) { return __int_as_float(0x4B400000 + m) - 12582912.f; }
 template <int T> __device__ __forceinline__ void oz_digits(long long I, float (&d)[T]) {
+  static_assert(T == 7, "four digits from the low 28 bits, three from the rest");
+  int x = (int)(I & 0xFFFFFFF);
 #pragma unroll
-  for (int t = T - 1; t >= 1; --t) {
-    const long long m = ((I + 64) & 127) - 64;
-    d[t] = (float)m;
-    I = (I - m) >> 7;
+  for (int t = T - 1; t >= 3; --t) {
+    const int m = ((x + 64) & 127) - 64;
+    d[t] = oz_small_float(m);
+    x = (x - m) >> 7;
   }
-  d[0] = (float)I;
+  x += (int)(I >> 28);
+#pragma unroll
+  for (int t = 2; t >= 1; --t) {
+    const int m = ((x + 64) & 127) - 64;
+    d[t] = oz_small_float(m);
+    x = (x - m) >> 7;
+  }
+  d[0] = oz_small_float(x);
 }
 
 __device__ __forceinline__ int oz_exponent(float m) { return m > 0.f ? ilogbf(m) + 1 : 0; }
@@ -348,42 +361,76 @@ __device__ __forceinline__ void put_bf16x2(uint16_t *dst, float a, float b) {
 }
 
 // digits of the rows of a complex matrix (K = 2 N_int real values per row, src[r][ld] complex),
-// times the Gamma-point weights (1 on the first len0 elements, 2 on the rest) when weighted;
-// one block of 256 threads per row, four elements per thread and iteration with their loads
-// issued together. dig: [T][rows][kpad], ex: [rows].
-template <int T>
+// times the Gamma-point weights (1 on the first len0 elements, 2 on the rest) when weighted.
+// dig: [T][rows][kpad], ex: [rows].
+// A row belongs to a cluster of CL CTAs of 256 threads, each with a CL-th of it: the elements are read
+// once (the first `keep` of a CTA's share stay in shared memory), the CTAs exchange their maxima
+// through distributed shared memory, and the digits are made from the kept copy. The floor is HBM:
+// 16 bytes read and 28 written per element. With a block per row that read it twice, and 64-bit integer
+// digits, 512 rows of 23,149 took 460 us (1.1 TB/s) and 3 rows of 8,455 43 us; here 120 us (4.3 TB/s) and
+// 5 us.
+__device__ __forceinline__ float pow2f(int k) { return __int_as_float((k + 127) << 23); }  // -126 <= k <= 127
+
+template <int T, int CL>
 __global__ void __launch_bounds__(256) k_oz_rows_df(const cplx<df64> *__restrict__ src, int ld, int nint, int len0, bool weighted,
-                                                    uint16_t *__restrict__ dig, int kpad, size_t plane, int *__restrict__ ex) {
+                                                    uint16_t *__restrict__ dig, int kpad, size_t plane, int *__restrict__ ex, int keep) {
   constexpr int U = 4;
-  const int r = blockIdx.x;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cplx<df64> *kept = reinterpret_cast<cplx<df64> *>(smraw);
+  __shared__ float cta_max;
+  const int r = blockIdx.x / CL, per = (nint + CL - 1) / CL;
+  const int b0 = (blockIdx.x % CL) * per, b1 = min(nint, b0 + per);
   const cplx<df64> *row = src + (size_t)r * ld;
   const cplx<df64> zero = mkc<df64>(df64(0.f, 0.f), df64(0.f, 0.f));
   float m = 0.f;
-  for (int e0 = threadIdx.x; e0 < nint; e0 += 256 * U) {
+  for (int e0 = b0 + (int)threadIdx.x; e0 < b1; e0 += 256 * U) {
     cplx<df64> v[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = e0 + 256 * u < nint ? row[e0 + 256 * u] : zero;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const float w = (weighted && e0 + 256 * u >= len0) ? 2.f : 1.f;
-      m = fmaxf(m, w * fmaxf(fabsf(v[u].x.hi), fabsf(v[u].y.hi)));
-    }
-  }
-  m = block_max256(m);
-  const int E = oz_exponent(m);
-  if (threadIdx.x == 0) ex[r] = E;
-  const int sh = 7 * T - E;
-  for (int e0 = threadIdx.x; e0 < nint; e0 += 256 * U) {
-    cplx<df64> v[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = e0 + 256 * u < nint ? row[e0 + 256 * u] : zero;
+    for (int u = 0; u < U; ++u) v[u] = e0 + 256 * u < b1 ? row[e0 + 256 * u] : zero;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int e = e0 + 256 * u;
-      if (e >= nint) break;
-      const int sw = sh + ((weighted && e >= len0) ? 1 : 0);
-      const long long Ix = __float2ll_rn(ldexpf(v[u].x.hi, sw)) + __float2ll_rn(ldexpf(v[u].x.lo, sw));
-      const long long Iy = __float2ll_rn(ldexpf(v[u].y.hi, sw)) + __float2ll_rn(ldexpf(v[u].y.lo, sw));
+      const float w = (weighted && e >= len0) ? 2.f : 1.f;
+      m = fmaxf(m, w * fmaxf(fabsf(v[u].x.hi), fabsf(v[u].y.hi)));
+      if (e < b1 && e - b0 < keep) kept[e - b0] = v[u];
+    }
+  }
+  m = block_max256(m);
+  if constexpr (CL > 1) {
+    if (threadIdx.x == 0) cta_max = m;
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    const uint32_t mine = tc::smem_u32(&cta_max);
+#pragma unroll
+    for (int k = 0; k < CL; ++k) {
+      uint32_t addr;
+      float o;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(mine), "r"(k));
+      asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(o) : "r"(addr) : "memory");
+      m = fmaxf(m, o);
+    }
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");  // every CTA has read the maxima
+  }
+  const int E = oz_exponent(m);
+  if (threadIdx.x == 0 && b0 == 0) ex[r] = E;
+  // scale by 2^(7T - E) in two exact steps (E reaches -148: one power of two would not be a float)
+  const int sh = 7 * T - E, s1 = sh / 2;
+  const float p1 = pow2f(s1), p2 = pow2f(sh - s1);
+  for (int e0 = b0 + (int)threadIdx.x; e0 < b1; e0 += 256 * U) {
+    cplx<df64> v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + 256 * u;
+      v[u] = zero;
+      if (e < b1) v[u] = e - b0 < keep ? kept[e - b0] : row[e];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = e0 + 256 * u;
+      if (e >= b1) break;
+      const float q2 = (weighted && e >= len0) ? 2.f * p2 : p2;
+      const long long Ix = __float2ll_rn(v[u].x.hi * p1 * q2) + __float2ll_rn(v[u].x.lo * p1 * q2);
+      const long long Iy = __float2ll_rn(v[u].y.hi * p1 * q2) + __float2ll_rn(v[u].y.lo * p1 * q2);
       float dx[T], dy[T];
       oz_digits<T>(Ix, dx);
       oz_digits<T>(Iy, dy);
@@ -391,6 +438,7 @@ __global__ void __launch_bounds__(256) k_oz_rows_df(const cplx<df64> *__restrict
       for (int t = 0; t < T; ++t) put_bf16x2(dig + t * plane + (size_t)r * kpad + 2 * e, dx[t], dy[t]);
     }
   }
+  if constexpr (CL > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // the same from FP64 rows (the projectors and orbitals, once per context)
@@ -421,51 +469,48 @@ __global__ void __launch_bounds__(256) k_oz_rows_f64(const cplx<double> *__restr
 
 // digits of the transpose of an FP64 matrix src[j][c] (j < nj rows, c < ncol columns, row stride
 // lds), each source row scaled by d[j] when d is given: output row c has K = nj values (over j)
-// and its own exponent. Blocks of 32 columns x 8 row lanes; dig: [T][ncol][kpad], ex: [ncol].
+// and its own exponent. A warp per column, lanes along j in pairs (4-byte stores), eight adjacent
+// columns a block (their warps share the 64 bytes of a row), UC pairs of loads in flight: the passes are
+// latency-bound. Blocks of 32 columns that walked j in steps of 8 took 125 us for 768 x 512 (16
+// blocks) and 31 us for 192 x 3; here 20 and 4 us. dig: [T][ncol][kpad], ex: [ncol].
 template <int T>
 __global__ void __launch_bounds__(256) k_oz_cols(const double *__restrict__ src, size_t lds, int nj, int ncol, const double *__restrict__ d,
                                                  uint16_t *__restrict__ dig, int kpad, size_t plane, int *__restrict__ ex) {
-  __shared__ double red[8][33];
-  __shared__ float tile[T][32][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int c0 = blockIdx.x * 32, c = c0 + tx;
+  constexpr int UC = 4;
+  const int lane = threadIdx.x & 31, c = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (c >= ncol) return;
+  auto value = [&](int j) { return j < nj ? src[(size_t)j * lds + c] * (d ? d[j] : 1.0) : 0.0; };
   double m = 0.0;
-  if (c < ncol)
-    for (int j = ty; j < nj; j += 8) m = fmax(m, fabs(src[(size_t)j * lds + c] * (d ? d[j] : 1.0)));
-  red[ty][tx] = m;
-  __syncthreads();
-  if (ty == 0) {
-    for (int w = 1; w < 8; ++w) m = fmax(m, red[w][tx]);
-    red[0][tx] = (double)oz_exponent(m);
-    if (c < ncol) ex[c] = oz_exponent(m);
+  for (int j0 = 2 * lane; j0 < nj; j0 += 64 * UC) {
+    double v[UC][2];
+#pragma unroll
+    for (int u = 0; u < UC; ++u) {
+      v[u][0] = value(j0 + 64 * u);
+      v[u][1] = value(j0 + 64 * u + 1);
+    }
+#pragma unroll
+    for (int u = 0; u < UC; ++u) m = fmax(m, fmax(fabs(v[u][0]), fabs(v[u][1])));
   }
-  __syncthreads();
-  const int E = (int)red[0][tx];
-  for (int j0 = 0; j0 < nj; j0 += 32) {
-    // rows j0 + ty + 8 i: thread (tx, ty) makes the digits of column c, then writes them transposed
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int E = oz_exponent(m);
+  if (lane == 0) ex[c] = E;
+  for (int j0 = 2 * lane; j0 < nj; j0 += 64 * UC) {
+    double v[UC][2];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int jj = ty + 8 * i, j = j0 + jj;
-      float dd[T];
-      double v = 0.0;
-      if (c < ncol && j < nj) v = src[(size_t)j * lds + c] * (d ? d[j] : 1.0);
-      oz_digits<T>(__double2ll_rn(ldexp(v, 7 * T - E)), dd);
-#pragma unroll
-      for (int t = 0; t < T; ++t) tile[t][tx][jj] = dd[t];
+    for (int u = 0; u < UC; ++u) {
+      v[u][0] = value(j0 + 64 * u);
+      v[u][1] = value(j0 + 64 * u + 1);
     }
-    __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int cc = ty + 8 * i, col = c0 + cc, j = j0 + tx;
-      if (col < ncol && j < nj) {
+    for (int u = 0; u < UC; ++u) {
+      const int j = j0 + 64 * u;
+      if (j >= nj) break;
+      float a[T], b[T];
+      oz_digits<T>(__double2ll_rn(ldexp(v[u][0], 7 * T - E)), a);
+      oz_digits<T>(__double2ll_rn(ldexp(v[u][1], 7 * T - E)), b);  // zero past the last row: kpad covers it
 #pragma unroll
-        for (int t = 0; t < T; ++t) {
-          const __nv_bfloat16 b = __float2bfloat16_rn(tile[t][cc][tx]);
-          dig[t * plane + (size_t)col * kpad + j] = __bfloat16_as_ushort(b);
-        }
-      }
+      for (int t = 0; t < T; ++t) put_bf16x2(dig + t * plane + (size_t)c * kpad + j, a[t], b[t]);
     }
-    __syncthreads();
   }
 }
 
@@ -505,6 +550,15 @@ int num_sms() {
   return nsm;
 }
 
+// K splits of the Gram: enough work items for the SMs, down to one chain (OZ_CHAIN stages) each, and at
+// most OZ_MAXCHAIN chains per split. With at least four chains a split the 192 x 3 products of the
+// 64^3 system ran in 16 CTAs of 66 stages (60 us); in 66 CTAs of 16 they take 26 us.
+int gram_splits(int tiles, int nst) {
+  int nsplit = std::max(1, (nst + OZ_CHAIN * OZ_MAXCHAIN - 1) / (OZ_CHAIN * OZ_MAXCHAIN));
+  while (tiles * nsplit < num_sms() && nst / (nsplit + 1) >= OZ_CHAIN) ++nsplit;
+  return nsplit;
+}
+
 template <int T, int EPI>
 void run_gemm(const OzMat &A, const OzMat &B, int K, OzArgs p, double *work, size_t work_cap, cudaStream_t st) {
   p.rowsA = A.rows;
@@ -514,11 +568,8 @@ void run_gemm(const OzMat &A, const OzMat &B, int K, OzArgs p, double *work, siz
   p.tilesA = (A.rows + OZ_M - 1) / OZ_M;
   p.tilesB = (B.rows + OZ_NB - 1) / OZ_NB;
   p.nst = (K + OZ_KS - 1) / OZ_KS;
-  // K splits: enough CTAs for the SMs, and at most OZ_MAXCHAIN chains per split
   const int tiles = p.tilesA * p.tilesB, nsm = num_sms();
-  int nsplit = std::max(1, (p.nst + OZ_CHAIN * OZ_MAXCHAIN - 1) / (OZ_CHAIN * OZ_MAXCHAIN));
-  if (EPI == OZ_GRAM)
-    while (tiles * nsplit < nsm && p.nst / (nsplit + 1) >= 4 * OZ_CHAIN) ++nsplit;
+  int nsplit = EPI == OZ_GRAM ? gram_splits(tiles, p.nst) : std::max(1, (p.nst + OZ_CHAIN * OZ_MAXCHAIN - 1) / (OZ_CHAIN * OZ_MAXCHAIN));
   p.per = (p.nst + nsplit - 1) / nsplit;
   nsplit = std::max(1, (p.nst + p.per - 1) / p.per);
   double *final_out = p.out;
@@ -548,6 +599,10 @@ void run_gemm(const OzMat &A, const OzMat &B, int K, OzArgs p, double *work, siz
 
 }  // namespace
 
+// elements of a CTA's share of a row that k_oz_rows_df keeps in shared memory (46 KB at the 96^3 system's
+// 23,149 over 8 CTAs; longer shares read the rest a second time)
+constexpr int kRowKeep = 4096;
+
 bool oz_enabled() {
   static const bool on = std::getenv("WDF_NO_OZ") == nullptr;
   return on && tc_enabled();
@@ -558,13 +613,44 @@ int oz_kpad(int K) { return ((K + OZ_KS - 1) / OZ_KS) * OZ_KS; }
 void set_oz_limits() {
   raise_smem_limit(k_oz_gemm<OZ_DIGITS, OZ_GRAM>, oz_smem<OZ_DIGITS>());
   raise_smem_limit(k_oz_gemm<OZ_DIGITS, OZ_LINCOMB>, oz_smem<OZ_DIGITS>());
+  raise_smem_limit(k_oz_rows_df<OZ_DIGITS, 1>, sizeof(cplx<df64>) * kRowKeep);
+  raise_smem_limit(k_oz_rows_df<OZ_DIGITS, 8>, sizeof(cplx<df64>) * kRowKeep);
 }
 
 void launch_oz_rows_df(const Geo &g, const cplx<df64> *src, int rows, bool weighted, const OzMat &out, cudaStream_t st) {
   if (rows <= 0) return;
-  launch("oz_slice", 64, k_oz_rows_df<OZ_DIGITS>, dim3(rows), dim3(256), 0, st, src, g.ld, g.nint, g.len0, weighted, out.dig, out.kpad,
-         out.plane, out.ex);
-  WDF_CUDA_TRY(cudaGetLastError());
+  // a cluster of 8 CTAs per row when a row is long, or rows are few and not short; else one CTA
+  constexpr int CL = 8;
+  const bool wide = g.nint >= 4096 || (rows < 2 * 152 && g.nint >= 1024);
+  const int share = wide ? (g.nint + CL - 1) / CL : g.nint, keep = std::min(share, kRowKeep);
+  const size_t sm = sizeof(cplx<df64>) * (size_t)keep;
+  if (!wide) {
+    launch("oz_slice", 64, k_oz_rows_df<OZ_DIGITS, 1>, dim3(rows), dim3(256), sm, st, src, g.ld, g.nint, g.len0, weighted, out.dig,
+           out.kpad, out.plane, out.ex, keep);
+    WDF_CUDA_TRY(cudaGetLastError());
+    return;
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)rows * CL);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = CL;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  const bool timed = t_prof && t_prof->bits == 64 && t_prof->target == "oz_slice";
+  if (timed) prof_record(st);
+  WDF_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_oz_rows_df<OZ_DIGITS, CL>, src, g.ld, g.nint, g.len0, weighted, out.dig, out.kpad, out.plane,
+                                  out.ex, keep));
+  if (timed) {
+    prof_record(st);
+    ++t_prof->count;
+    t_prof->blocks += (long long)rows * CL;
+  }
 }
 
 void launch_oz_rows_f64(const Geo &g, const cplx<double> *src, int rows, bool weighted, const OzMat &out, cudaStream_t st) {
@@ -576,7 +662,7 @@ void launch_oz_rows_f64(const Geo &g, const cplx<double> *src, int rows, bool we
 
 void launch_oz_cols(const double *src, size_t lds, int nj, int ncol, const double *d, const OzMat &out, cudaStream_t st) {
   if (ncol <= 0) return;
-  launch("oz_slice", 64, k_oz_cols<OZ_DIGITS>, dim3((ncol + 31) / 32), dim3(256), 0, st, src, lds, nj, ncol, d, out.dig, out.kpad,
+  launch("oz_slice", 64, k_oz_cols<OZ_DIGITS>, dim3((ncol + 7) / 8), dim3(256), 0, st, src, lds, nj, ncol, d, out.dig, out.kpad,
          out.plane, out.ex);
   WDF_CUDA_TRY(cudaGetLastError());
 }
@@ -584,8 +670,7 @@ void launch_oz_cols(const double *src, size_t lds, int nj, int ncol, const doubl
 size_t oz_gram_work_doubles(int na, int nb, int K) {
   const int nst = (K + OZ_KS - 1) / OZ_KS;
   const int tiles = ((na + OZ_M - 1) / OZ_M) * ((nb + OZ_NB - 1) / OZ_NB);
-  int nsplit = std::max(1, (nst + OZ_CHAIN * OZ_MAXCHAIN - 1) / (OZ_CHAIN * OZ_MAXCHAIN));
-  while (tiles * nsplit < num_sms() && nst / (nsplit + 1) >= 4 * OZ_CHAIN) ++nsplit;
+  const int nsplit = gram_splits(tiles, nst);
   return nsplit > 1 ? (size_t)nsplit * na * nb : 0;
 }
 
