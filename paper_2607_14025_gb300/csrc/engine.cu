@@ -1256,8 +1256,8 @@ template <typename T> static void autotune_vloc(wdf_ctx *c, FftCtx<T> &f, const 
       if (!plane_variant_available<T>(f, v)) continue;
       // the line-resident kernel beats the Stockham, generic and one-task-per-thread kernels at every
       // size it exists for (FP32 1.6-3.5x, double-float 1.5-3.5x over the best of them at 24^2 ... 96^2):
-      // only the register and persistent FP32 kernels are timed against it
-      if (lines && (v == 2 || v == 3 || v == 4 || v == 6)) continue;
+      // only the register and persistent FP32 kernels are timed against it (and variant 6 is it)
+      if (lines && (v == 2 || v == 3 || v == 4 || (v == 8 && plane_variant_available<T>(f, 6)))) continue;
       f.vloc_variant = v;
       launch_plane<T>(f, OP_VLOC, nblk, pa, st);  // warm-up
       WDF_CUDA_TRY(cudaEventRecord(e0, st));
@@ -1283,7 +1283,7 @@ template <typename T> static void autotune_vloc(wdf_ctx *c, FftCtx<T> &f, const 
   cbuf.release();
   f.vloc_variant = bestv;
   if (std::getenv("WDF_TRACE"))
-    fprintf(stderr, "[wdf] V_loc plane kernel (%d-bit): variant %d (1 register, 2 Stockham, 3 generic, 4 two-thread register, 5 persistent, 6 double-float, 7 two-thread persistent, 8 line-resident), %.3f ms per %d pairs\n",
+    fprintf(stderr, "[wdf] V_loc plane kernel (%d-bit): variant %d (1 register, 2 Stockham, 3 generic, 4 two-thread register, 5 persistent, 6 double-float 64 x 64, 8 line-resident), %.3f ms per %d pairs\n",
             bits_of<T>(), bestv, best / 3, nblk);
 }
 

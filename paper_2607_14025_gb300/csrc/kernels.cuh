@@ -20,9 +20,9 @@ template <typename T> struct FftCtx {
   int vloc_variant = 0;            // V_loc plane kernel: 0 default order, 1 register, 2 Stockham, 3 generic,
                                    // 4 register with two threads per line (n1 = n2 = 64), 5 persistent
                                    // with bulk copies (64 x 64 planes with a full disk), 6 double-float
-                                   // one task per thread (64 x 64), 7 persistent with two threads per
-                                   // line (96 x 96 planes with a full disk), 8 whole lines in the
-                                   // registers of a few lanes (float and double-float)
+                                   // 64 x 64 (line-resident within the band it takes, else one task
+                                   // per thread), 7 unused, 8 whole lines in the registers of a few
+                                   // lanes
   const T *vgroup = nullptr;       // float: V_loc in the line-resident kernels' order (lines_group_vloc)
   int *err = nullptr;              // device flag set by a kernel whose bounded wait expired
 };
@@ -50,8 +50,7 @@ bool plane_fast_supported(int n1, int n2);
 template <typename T> void set_plane_fast_limits(const Geo &g);
 template <typename T> bool launch_plane_fast(const FftCtx<T> &f, int op, int nblk, const PlaneArgs<T> &pa, cudaStream_t st);
 // whether V_loc plane variant v (1 register, 2 Stockham, 3 generic, 4 two-thread register,
-// 5 persistent with bulk copies, 6 double-float one task per thread, 7 persistent with two threads
-// per line, 8 line-resident) exists
+// 5 persistent with bulk copies, 6 double-float 64 x 64, 8 line-resident) exists
 template <typename T> bool plane_variant_available(const FftCtx<T> &f, int v);
 constexpr int kPlaneVariants = 8;  // variants are numbered 1 .. kPlaneVariants
 // whether the orbital sum of the density response runs as G2R transforms + k_orbital_sum
@@ -65,10 +64,6 @@ template <typename R> void launch_fill(R *x, size_t count, double value, cudaStr
 bool plane_pipe_available(const Geo &g, const int *err);
 void set_plane_pipe_limits(const Geo &g);
 bool launch_plane_pipe(const FftCtx<float> &f, int npair, const PlaneArgs<float> &pa, cudaStream_t st);
-// persistent FP32 V_loc plane kernel with two threads per line (plane_pipe2.cu; 96 x 96 planes)
-bool plane_pipe2_available(const Geo &g, const int *err);
-void set_plane_pipe2_limits(const Geo &g);
-bool launch_plane_pipe2(const FftCtx<float> &f, int npair, const PlaneArgs<float> &pa, cudaStream_t st);
 // compile-time Stockham plane kernels for the further sizes (plane_more_*.cu): float, and
 // double-float in two size groups; false when the size is not in the group
 bool launch_plane_more_f32(const FftCtx<float> &f, int op, int nblk, const PlaneArgs<float> &pa, cudaStream_t st);

@@ -349,10 +349,13 @@ template <typename T> static void set_lines_limits(const Geo &g) {
   }
 #undef X
 }
-// the line-resident kernel runs this context's plane operations: chosen by the setup timing, or FP64
-// without a timing of its own (the ground state, and H x in a double-float context)
+// the line-resident kernel runs this context's plane operations: chosen by the setup timing; as the
+// double-float 64 x 64 kernel (variant 6, which keeps the one-task-per-thread kernel for wider bands);
+// or FP64 without a timing of its own (the ground state, and H x in a double-float context)
 template <typename T> static bool lines_chosen(const FftCtx<T> &f) {
-  return f.vloc_variant == 8 || (std::is_same<T, double>::value && f.vloc_variant == 0 && lines_available(f.g, f.jidx));
+  if (f.vloc_variant == 8) return true;
+  const int other = std::is_same<T, df64>::value ? 6 : std::is_same<T, double>::value ? 0 : -1;
+  return f.vloc_variant == other && lines_available(f.g, f.jidx);
 }
 template <typename T> static bool launch_lines(const FftCtx<T> &f, int op, int nblk, const PlaneArgs<T> &pa, cudaStream_t st) {
 #define X(NAME) launch_##NAME(f, op, nblk, pa, st) ||
@@ -377,7 +380,6 @@ template <typename T> void set_plane_fast_limits(const Geo &g) {
   if (std::is_same<T, float>::value && g.n1 == g.n2) {
     set_plane_reg_limits(g);
     set_plane_pipe_limits(g);
-    set_plane_pipe2_limits(g);
   }
   if (std::is_same<T, df64>::value) set_plane_df_limits(g);
   set_lines_limits<T>(g);
@@ -398,9 +400,9 @@ template <typename T> void set_plane_fast_limits(const Geo &g) {
 template <typename T> bool launch_plane_fast(const FftCtx<T> &f, int op, int nblk, const PlaneArgs<T> &pa, cudaStream_t st) {
   const int v = op == OP_VLOC ? f.vloc_variant : 0;  // chosen at setup by timing (0: this order)
   if constexpr (std::is_same<T, df64>::value) {
-    // the double-float 64 x 64 kernel: V_loc when the setup timing chose it, the product and the
-    // orbital sum whenever it exists
-    const bool use = op == OP_VLOC ? v == 6 : ((op == OP_PROD_R2G && f.vloc_variant != 8) || op == OP_ACCUM);
+    // the one-task-per-thread 64 x 64 kernel: the orbital sum whenever it exists, V_loc (variant 6) and
+    // the product for bands that the line-resident kernel does not take
+    const bool use = op == OP_ACCUM || (!lines_chosen(f) && (op == OP_VLOC ? v == 6 : op == OP_PROD_R2G));
     if (use && launch_plane_df(f, op, nblk, pa, st)) return true;
   }
   // the orbital sum of the density response keeps two register blocks across its loop and
@@ -413,8 +415,7 @@ template <typename T> bool launch_plane_fast(const FftCtx<T> &f, int op, int nbl
   // kernel won it (large double-float planes), they use the generic kernel too
   if (op != OP_VLOC && f.vloc_variant == 3) return false;
   if constexpr (std::is_same<T, float>::value) {
-    if (op == OP_VLOC && v == 5 && launch_plane_pipe(f, nblk, pa, st)) return true;
-    if (op == OP_VLOC && v == 7 && launch_plane_pipe2(f, nblk, pa, st)) return true;
+    if (op == OP_VLOC && v == 5 && f.vgroup && launch_plane_pipe(f, nblk, pa, st)) return true;
     if (op == OP_VLOC && v == 4 && launch_plane_reg2(f, nblk, pa, st)) return true;
     if (op == OP_VLOC && v != 2 && launch_plane_reg(f, nblk, pa, st)) return true;
   }
@@ -437,8 +438,7 @@ template <typename T> bool plane_variant_available(const FftCtx<T> &f, int v) {
   if (v == 3) return true;
   if (f.jidx == nullptr) return false;
   if (v == 4) return std::is_same<T, float>::value && reg_plane_enabled() && g.n1 == 64 && g.n2 == 64;
-  if (v == 5) return std::is_same<T, float>::value && plane_pipe_available(g, f.err);
-  if (v == 7) return std::is_same<T, float>::value && plane_pipe2_available(g, f.err);
+  if (v == 5) return std::is_same<T, float>::value && f.vgroup && plane_pipe_available(g, f.err);
   if (v == 8) return (!std::is_same<T, float>::value || f.vgroup) && lines_available(g, f.jidx);
   if (v == 6) return std::is_same<T, df64>::value && plane_df_available(g, f.jidx);
   if (v == 2) return plane_fast_supported(g.n1, g.n2) || (!std::is_same<T, double>::value && plane_more_supported(g.n1, g.n2));
