@@ -156,7 +156,7 @@ void launch_zpass_g2r(const FftCtx<T> &f, const cplx<T> *X, int nvec, cplx<T> *c
   if constexpr (has_more<T>())
     if (zpass_more_g2r<T>(f, X, nvec, cb, st)) return;
   dim3 grid((nvec + 1) / 2, (f.g.K + kZCols - 1) / kZCols);
-  launch("zpass_g2r", bits_of<T>(), k_zpass_g2r<T, false, 0>, dim3(grid), dim3(kThreads), zpass_smem<T>(f.g), st, X, nvec, f.g, f.P3,
+  launch_pdl("zpass_g2r", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_g2r<T, false, 0>, dim3(grid), dim3(kThreads), zpass_smem<T>(f.g), st, X, nvec, f.g, f.P3,
          f.tw3, cb, PDir<T>());
   WDF_CUDA_TRY(cudaGetLastError());
 }
@@ -168,7 +168,7 @@ void launch_zpass_g2r_dir(const FftCtx<T> &f, const PDir<T> &d, int nvec, cplx<T
   if constexpr (has_more<T>())
     if (zpass_more_g2r_dir<T>(f, d, nvec, cb, st)) return;
   dim3 grid((nvec + 1) / 2, (f.g.K + kZCols - 1) / kZCols);
-  launch("zpass_g2r", bits_of<T>(), k_zpass_g2r<T, true, 0>, dim3(grid), dim3(kThreads), zpass_smem<T>(f.g), st,
+  launch_pdl("zpass_g2r", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_g2r<T, true, 0>, dim3(grid), dim3(kThreads), zpass_smem<T>(f.g), st,
          (const cplx<T> *)d.p, nvec, f.g, f.P3, f.tw3, cb, d);
   WDF_CUDA_TRY(cudaGetLastError());
 }
@@ -181,9 +181,9 @@ void launch_zpass_r2g(const FftCtx<T> &f, int epi, const cplx<T> *cb, int nvec, 
     if (zpass_more_r2g<T>(f, epi, cb, nvec, ea, st)) return;
   dim3 grid((nvec + 1) / 2, (f.g.K + kZCols - 1) / kZCols);
   const size_t sm = zpass_smem<T>(f.g);
-  if (epi == EPI_STORE) launch("zpass_r2g", bits_of<T>(), k_zpass_r2g<T, EPI_STORE, 0>, dim3(grid), dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
-  else if (epi == EPI_HSHIFT) launch("zpass_r2g", bits_of<T>(), k_zpass_r2g<T, EPI_HSHIFT, 0>, dim3(grid), dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
-  else launch("zpass_r2g", bits_of<T>(), k_zpass_r2g<T, EPI_DRHO, 0>, dim3(grid), dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
+  if (epi == EPI_STORE) launch_pdl("zpass_r2g", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_r2g<T, EPI_STORE, 0>, dim3(grid), dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
+  else if (epi == EPI_HSHIFT) launch_pdl("zpass_r2g", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_r2g<T, EPI_HSHIFT, 0>, dim3(grid), dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
+  else launch_pdl("zpass_r2g", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_r2g<T, EPI_DRHO, 0>, dim3(grid), dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
   WDF_CUDA_TRY(cudaGetLastError());
 }
 

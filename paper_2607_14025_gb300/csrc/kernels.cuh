@@ -141,7 +141,8 @@ template <typename T>
 void launch_lincomb(const Geo &g, cplx<T> *Y, int ny, const cplx<T> *U, int nu, const double *C, int ldc,
                     const double *d, double c0, cudaStream_t st);
 // launch_lincomb plus partial inner products <P_s, Y_s> of the results, written to
-// part[s * lincomb_dot_chunks(g) + block]; returns false (nothing launched) for ny <= 8
+// part[s * lincomb_dot_chunks(g) + block]; returns false (nothing launched) for ny <= 8 in FP32 and
+// double-float
 template <typename T>
 bool launch_lincomb_dot(const Geo &g, cplx<T> *Y, int ny, const cplx<T> *U, int nu, const double *C, int ldc, const double *d,
                         double c0, const cplx<T> *P, double *part, cudaStream_t st);

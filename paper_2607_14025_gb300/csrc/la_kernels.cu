@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(256) k_lincomb(Geo g, cplx<T> *__restrict__ Y,
   }
 }
 
-// FP64 linear combinations into more than 8 vectors: a warp owns 32 elements (a block LE = 128) of VQ
+// FP64 linear combinations: a warp owns 32 elements (a block LE = 128) of VQ
 // vectors, each lane one element, rows of U read once per VQ vectors (coalesced, from L2), the
 // scaled coefficients staged LJ64 rows at a time. As for the Gram products only the FMAs count: at
 // most VQ - 1 padded vectors and enough blocks for the 152 SMs. VQ = 4 until the vectors alone
@@ -617,14 +617,18 @@ __global__ void __launch_bounds__(128) k_lincomb_f64(Geo g, double2 *__restrict_
 static void launch_lincomb_f64(const Geo &g, double2 *Y, int ny, const double2 *U, int nu, const double *C, int ldc, const double *d,
                                double c0, const double2 *P, double *part, cudaStream_t st) {
   const int ne = (g.nint + LE - 1) / LE;
-  if ((long)ne * ((ny + 7) / 8) >= 4 * 152)
-    launch("lincomb", 64, k_lincomb_f64<8>, dim3((ny + 7) / 8, ne), dim3(128), 0, st, g, Y, ny, U, nu, C, ldc, d, c0, P, part);
-  else
-    launch("lincomb", 64, k_lincomb_f64<4>, dim3((ny + 3) / 4, ne), dim3(128), 0, st, g, Y, ny, U, nu, C, ldc, d, c0, P, part);
+  auto go = [&](auto kernel, int vq) {
+    launch("lincomb", 64, kernel, dim3((ny + vq - 1) / vq, ne), dim3(128), 0, st, g, Y, ny, U, nu, C, ldc, d, c0, P, part);
+  };
+  if (ny == 1) go(k_lincomb_f64<1>, 1);
+  else if (ny == 2) go(k_lincomb_f64<2>, 2);
+  else if ((long)ne * ((ny + 7) / 8) >= 4 * 152) go(k_lincomb_f64<8>, 8);
+  else go(k_lincomb_f64<4>, 4);
   WDF_CUDA_TRY(cudaGetLastError());
 }
 
-// Linear combinations into at most 8 vectors: each thread owns one element of every output.
+// FP32 and double-float linear combinations into at most 8 vectors: each thread owns one element of every
+// output.
 template <typename T, typename Acc>
 __global__ void __launch_bounds__(256) k_lincomb_narrow(Geo g, cplx<T> *__restrict__ Y, int ny, const cplx<T> *__restrict__ U, int nu,
                                                        const double *__restrict__ C, int ldc, const double *__restrict__ d, double c0) {
@@ -661,15 +665,11 @@ template <typename T>
 void launch_lincomb(const Geo &g, cplx<T> *Y, int ny, const cplx<T> *U, int nu, const double *C, int ldc, const double *d,
                     double c0, cudaStream_t st) {
   if (ny <= 0) return;
-  if (ny <= kNarrow) {
-    typedef typename std::conditional<std::is_same<T, float>::value, float, T>::type AccN;
-    launch("lincomb", bits_of<T>(), k_lincomb_narrow<T, AccN>, dim3((g.nint + 255) / 256), dim3(256), 0, st, g, Y, ny, U, nu, C, ldc,
-           d, c0);
-    WDF_CUDA_TRY(cudaGetLastError());
-    return;
-  }
   if constexpr (std::is_same<T, double>::value) {
     launch_lincomb_f64(g, Y, ny, U, nu, C, ldc, d, c0, nullptr, nullptr, st);
+  } else if (ny <= kNarrow) {
+    launch("lincomb", bits_of<T>(), k_lincomb_narrow<T, T>, dim3((g.nint + 255) / 256), dim3(256), 0, st, g, Y, ny, U, nu, C, ldc, d, c0);
+    WDF_CUDA_TRY(cudaGetLastError());
   } else {
     dim3 grid((g.nint + LE - 1) / LE, (ny + LS - 1) / LS);
     launch("lincomb", bits_of<T>(), k_lincomb<T, T>, dim3(grid), dim3(256), 0, st, g, Y, ny, U, nu, C, ldc, d, c0,
@@ -683,7 +683,7 @@ int lincomb_dot_chunks(const Geo &g) { return (g.nint + LE - 1) / LE; }
 template <typename T>
 bool launch_lincomb_dot(const Geo &g, cplx<T> *Y, int ny, const cplx<T> *U, int nu, const double *C, int ldc, const double *d,
                         double c0, const cplx<T> *P, double *part, cudaStream_t st) {
-  if (ny <= kNarrow) return false;  // the narrow kernel has no dot epilogue
+  if (ny <= kNarrow && !std::is_same<T, double>::value) return false;  // the narrow kernel has no dot epilogue
   if constexpr (std::is_same<T, double>::value) {
     launch_lincomb_f64(g, Y, ny, U, nu, C, ldc, d, c0, P, part, st);
   } else {
@@ -778,13 +778,32 @@ void launch_cg_start(const Geo &g, const cplx<T> *r, cplx<T> *p, const T *kprec,
   WDF_CUDA_TRY(cudaGetLastError());
 }
 
-// block_sum with the result in every thread
-static __device__ double block_sum_all(double v) {
-  __shared__ double bc;
-  v = block_sum(v);
-  if (threadIdx.x == 0) bc = v;
+// block sums of a 256-thread block, one barrier: of one value in every thread (red: 8 doubles that the
+// block does not use otherwise), and of three values in thread 0
+static __device__ double block_sum_all(double v, double *red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  return bc;
+  double s = 0.0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) s += red[w];
+  return s;
+}
+static __device__ void block_sum3(double (&v)[3], bool third, double (*red)[8]) {
+  for (int o = 16; o > 0; o >>= 1) {
+    v[0] += __shfl_down_sync(0xffffffffu, v[0], o);
+    v[1] += __shfl_down_sync(0xffffffffu, v[1], o);
+    if (third) v[2] += __shfl_down_sync(0xffffffffu, v[2], o);
+  }
+  if ((threadIdx.x & 31) == 0)
+    for (int q = 0; q < 3; ++q) red[q][threadIdx.x >> 5] = v[q];
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int q = 0; q < 3; ++q) {
+      v[q] = 0.0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) v[q] += red[q][w];
+    }
 }
 
 // One CG update per launch: alpha from the partial sums of <p, A p>, x += alpha p, r -= alpha A p, the
@@ -821,7 +840,7 @@ __device__ __forceinline__ void upd_k(float2 v, float (&k)[2]) {
 __device__ __forceinline__ void upd_k(double v, double (&k)[1]) { k[0] = v; }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_cg_update(Geo g, cplx<T> *__restrict__ x, cplx<T> *__restrict__ r, const cplx<T> *__restrict__ p,
+__global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict__ x, cplx<T> *__restrict__ r, const cplx<T> *__restrict__ p,
                                                   const cplx<T> *__restrict__ Ap, const T *__restrict__ kprec, CgState s, int nchunk,
                                                   int chunk, const double *__restrict__ dots, int ndot, int maxiter, int which) {
   typedef PartAcc<T> A;
@@ -829,7 +848,9 @@ __global__ void __launch_bounds__(256) k_cg_update(Geo g, cplx<T> *__restrict__ 
   typedef typename UpdVec<T>::K KV;
   constexpr int E = UpdVec<T>::E, UB = 2, STEP = 256 * E * UB;
   const int i = blockIdx.x, c = blockIdx.y;
-  __shared__ int last;
+  __shared__ double redp[8], red3[3][8];
+  pdl_begin();
+  pdl_wait();
   if (i == 0 && c == 0 && threadIdx.x == 0) s.nactive[which ^ 1] = 0;  // the next launch's count
   if (!s.active[i]) return;
   // learned table: also <r, K_TPA r> while the solve is on its learned row (for a restart)
@@ -856,12 +877,13 @@ __global__ void __launch_bounds__(256) k_cg_update(Geo g, cplx<T> *__restrict__ 
   load(e);
   double pap = 0.0;
   for (int k = threadIdx.x; k < ndot; k += blockDim.x) pap += dots[(size_t)i * ndot + k];
-  pap = block_sum_all(pap);
+  const double rz = s.rz[i];
+  pap = block_sum_all(pap, redp);
   if (!(pap > 0.0)) {  // breakdown: keep the current iterate (every block of the row sees the same sum)
     if (c == 0 && threadIdx.x == 0) s.active[i] = 0;
     return;
   }
-  const T al = (T)(s.rz[i] / pap);
+  const T al = (T)(rz / pap);
   A vrz = 0, vrr = 0, vr3 = 0;
   for (; e < e1; e += STEP, load(e)) {
 #pragma unroll
@@ -895,41 +917,39 @@ __global__ void __launch_bounds__(256) k_cg_update(Geo g, cplx<T> *__restrict__ 
       *reinterpret_cast<V *>(r + o + eu) = upd_vec(re);
     }
   }
-  const double brz = block_sum((double)vrz);
-  const double brr = block_sum((double)vrr);
-  const double br3 = fb ? block_sum((double)vr3) : 0.0;
-  if (threadIdx.x == 0) {
-    s.part1[(size_t)i * nchunk + c] = brz;
-    s.part2[(size_t)i * nchunk + c] = brr;
-    if (fb) s.part3[(size_t)i * nchunk + c] = br3;
+  double sum[3] = {(double)vrz, (double)vrr, (double)vr3};
+  block_sum3(sum, fb, red3);
+  if (threadIdx.x != 0) return;
+  if (nchunk > 1) {  // the last block of the row to arrive adds the chunks in order
+    s.part1[(size_t)i * nchunk + c] = sum[0];
+    s.part2[(size_t)i * nchunk + c] = sum[1];
+    if (fb) s.part3[(size_t)i * nchunk + c] = sum[2];
     __threadfence();
-    last = atomicAdd(&s.arrived[i], 1) == nchunk - 1;
+    if (atomicAdd(&s.arrived[i], 1) != nchunk - 1) return;
+    __threadfence();
+    s.arrived[i] = 0;
+    sum[0] = sum[1] = sum[2] = 0.0;
+    for (int k = 0; k < nchunk; ++k) {
+      sum[0] += __ldcg(s.part1 + (size_t)i * nchunk + k);
+      sum[1] += __ldcg(s.part2 + (size_t)i * nchunk + k);
+      if (fb) sum[2] += __ldcg(s.part3 + (size_t)i * nchunk + k);
+    }
   }
-  __syncthreads();
-  if (!last || threadIdx.x != 0) return;
-  __threadfence();
-  s.arrived[i] = 0;
-  const volatile double *q1 = s.part1 + (size_t)i * nchunk, *q2 = s.part2 + (size_t)i * nchunk, *q3 = s.part3 + (size_t)i * nchunk;
-  double a = 0.0, b = 0.0;
-  for (int k = 0; k < nchunk; ++k) a += q1[k];
-  for (int k = 0; k < nchunk; ++k) b += q2[k];
+  const double a = sum[0], b = sum[1];
   const int it = s.iters[i] + 1;
   s.iters[i] = it;
   s.rr[i] = b;
-  const double beta = a / s.rz[i];
   s.rz[i] = a;
-  s.rz_new[i] = beta;
+  s.rz_new[i] = a / rz;  // beta
   if (b <= s.thr[i] || it >= maxiter || !(b == b)) {
     s.active[i] = 0;
     return;
   }
   atomicAdd(&s.nactive[which], 1);
-  if (s.krow && s.krow[i] < s.nocc && it - s.it_ref[i] >= 5) {
+  if (fb && it - s.it_ref[i] >= 5) {
     if (b > 0.81 * s.rr_ref[i]) {  // stalled on the learned row: TPA from the current iterate
-      double c3 = 0.0;
-      for (int k = 0; k < nchunk; ++k) c3 += q3[k];
       s.krow[i] = s.vorig[i] + s.nocc;
-      s.rz[i] = c3;
+      s.rz[i] = sum[2];
       s.rz_new[i] = 0.0;  // beta = 0: p = K_TPA r
       atomicAdd(s.nfb, 1);
     }
@@ -946,7 +966,7 @@ void launch_cg_update(const Geo &g, cplx<T> *x, cplx<T> *r, const cplx<T> *p, co
   // 152 SMs twice over, so that a block's start and sums weigh less
   const int chunk = (long)n * ((g.nint + 4 * DCHUNK - 1) / (4 * DCHUNK)) >= 8 * 152 ? 4 * DCHUNK : DCHUNK;
   const int nchunk = (g.nint + chunk - 1) / chunk;
-  launch("cg_update", bits_of<T>(), k_cg_update<T>, dim3(n, nchunk), dim3(256), 0, st, g, x, r, p, Ap, kprec, s, nchunk, chunk, dots, ndot,
+  launch_pdl("cg_update", bits_of<T>(), (long long)n * nchunk, k_cg_update<T>, dim3(n, nchunk), dim3(256), 0, st, g, x, r, p, Ap, kprec, s, nchunk, chunk, dots, ndot,
          maxiter, which);
   WDF_CUDA_TRY(cudaGetLastError());
 }

@@ -264,6 +264,7 @@ __global__ void __launch_bounds__(32 * Lines<T, N>::W, Lines<T, N>::B)
   const int nx = g.nxact, xmax = g.xmax, ldcb = g.ldcb;
   const int u0 = blockIdx.x * ppb, np = min(ppb, nunits - u0);
   Gx *cb = pa.cb + (size_t)u0 * ldcb;
+  pdl_begin();
   if constexpr (L > 1)
     for (int i = t; i < N; i += TH) tw[i] = O::get(twg[i]);
   // the tile's columns between the occupied ones and the compile-time band read as zero
@@ -271,6 +272,7 @@ __global__ void __launch_bounds__(32 * Lines<T, N>::W, Lines<T, N>::B)
     const int gap = PITCH - nx;
     for (int i = t; i < np * N * gap; i += TH) tile[(i / gap) * PITCH + xmax + 1 + i % gap] = O::zero();
   }
+  pdl_wait();
   if constexpr (STAGE) {
     if (OP != OP_PROD_R2G) {
       const float4 *s = reinterpret_cast<const float4 *>(cb);
@@ -419,7 +421,7 @@ void lines_launch_op(const char *cls, const FftCtx<T> &f, int npair, const Plane
   // plane (8 solves on 24 x 24: 96 units, 12 blocks of 8 planes against 96 of one)
   const int ppb = std::max(1, std::min(D::P, (nunits + 152 * D::B - 1) / (152 * D::B)));
   const dim3 grid((unsigned)((nunits + ppb - 1) / ppb));
-  launch_units(cls, bits_of<T>(), nunits, k_plane_lines<T, N, OP>, grid, dim3(32 * D::W), lines_smem<T, N>(f.g, ppb), st, f.g, f.tw1, f.jidx,
+  launch_pdl(cls, bits_of<T>(), nunits, k_plane_lines<T, N, OP>, grid, dim3(32 * D::W), lines_smem<T, N>(f.g, ppb), st, f.g, f.tw1, f.jidx,
                a, nunits, ppb);
   WDF_CUDA_TRY(cudaGetLastError());
 }

@@ -83,6 +83,8 @@ __global__ void __launch_bounds__(PipeShape<N, XM>::threads, PipeShape<N, XM>::b
   uint64_t *bar = reinterpret_cast<uint64_t *>(tiles + 2 * N * NX);  // 3 (8-byte aligned as the tiles are)
   const int t = threadIdx.x, half = t < CT ? 0 : t < 2 * CT ? 1 : 2, l = t - half * CT;
   const long G = gridDim.x, u0 = blockIdx.x;
+  pdl_begin();
+  pdl_wait();
   if (u0 >= nunits) return;
   const int cnt = (int)((nunits - 1 - u0) / G) + 1;
   const uint32_t bytes = (uint32_t)ldcb * (uint32_t)sizeof(float2);
@@ -217,7 +219,7 @@ template <int N, int XM> void pipe_launch(const FftCtx<float> &f, int npair, con
   const long grid = std::min<long>(nunits, (long)nsm * per_sm);
   PlaneArgs<float> a = pa;
   a.field = f.vgroup;
-  launch_units("plane_vloc", 32, nunits, k_plane_pipe<N, XM>, dim3((unsigned)grid), dim3(TH), sm, st, f.g, f.jidx, a, nunits, f.err);
+  launch_pdl("plane_vloc", 32, nunits, k_plane_pipe<N, XM>, dim3((unsigned)grid), dim3(TH), sm, st, f.g, f.jidx, a, nunits, f.err);
   WDF_CUDA_TRY(cudaGetLastError());
 }
 

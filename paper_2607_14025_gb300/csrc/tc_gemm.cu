@@ -104,8 +104,10 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram_tc(const __grid_consta
     }
     tc::fence_mbar_init();
   }
+  pdl_begin();
   if (warp == 0) tc::tmem_alloc(slot, 512);
   tc::fence_before_sync();
+  pdl_wait();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *slot;
@@ -217,35 +219,43 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram_tc(const __grid_consta
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
-// Cd[s][j] = d_j sum over the splits of S[j][s] (j < na, else 0), hi and lo parts, through a 32 x 32
-// shared tile: the K splits of the Gram are added here, where they are read anyway
-__global__ void k_tc_coef(const double *__restrict__ S, int nsplit, size_t stride, int ldc, const double *__restrict__ d, int na, int nb,
-                          int kp, float *__restrict__ hi, float *__restrict__ lo) {
-  __shared__ float tile[32][33];
-  const int j0 = blockIdx.y * 32, s0 = blockIdx.x * 32;
-  {  // four rows of S per thread (blockDim.y = 8), their splits' loads in flight together
-    const int s = s0 + threadIdx.x;
-    const double *q = S + (size_t)(j0 + threadIdx.y) * ldc + s;
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
-    bool on[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) on[u] = s < nb && j0 + (int)threadIdx.y + 8 * u < na;
+// Cd[s][j] = d_j sum over the splits of S[j][s] (j < na, else 0), hi and lo parts: the K splits of the
+// Gram are added here, where they are read anyway. A block of 32 x 8 threads makes 4 rows of S x 32
+// solves, its 8 thread rows every eighth split: latency-bound for the many splits of a small system
+// (51 splits of 36 x 24: 16 us with a thread adding all splits of its outputs, 4.6 us here).
+__global__ void __launch_bounds__(256) k_tc_coef(const double *__restrict__ S, int nsplit, size_t stride, int ldc,
+                                                 const double *__restrict__ d, int na, int nb, int kp, float *__restrict__ hi,
+                                                 float *__restrict__ lo) {
+  __shared__ double red[8][4][33];
+  __shared__ float tile[4][33];
+  const int tx = threadIdx.x, ty = threadIdx.y, t = ty * 32 + tx;
+  const int j0 = blockIdx.y * 4, s0 = blockIdx.x * 32;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  pdl_begin();
+  pdl_wait();
+  if (s0 + tx < nb) {
+    const double *q = S + (size_t)j0 * ldc + s0 + tx;
 #pragma unroll 4
-    for (int k = 0; k < nsplit; ++k)
+    for (int k = ty; k < nsplit; k += 8)
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        if (on[u]) a[u] += q[k * stride + (size_t)(8 * u) * ldc];
+        if (j0 + u < na) a[u] += q[k * stride + (size_t)u * ldc];
+  }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int j = j0 + threadIdx.y + 8 * u;
-      tile[threadIdx.y + 8 * u][threadIdx.x] = on[u] ? (float)(a[u] * (d ? d[j] : 1.0)) : 0.f;
-    }
+  for (int u = 0; u < 4; ++u) red[ty][u][tx] = a[u];
+  __syncthreads();
+  if (t < 128) {
+    const int u = t >> 5, j = j0 + u;
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v += red[w][u][tx];
+    tile[u][tx] = j < na ? (float)(v * (d ? d[j] : 1.0)) : 0.f;
   }
   __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int s = s0 + r, j = j0 + threadIdx.x;
+  if (t < 128) {
+    const int u = t & 3, s = s0 + (t >> 2), j = j0 + u;
     if (s < nb && j < kp) {
-      const float v = tile[threadIdx.x][r];
+      const float v = tile[u][t >> 2];
       hi[(size_t)s * kp + j] = v;
       lo[(size_t)s * kp + j] = tc::tf32_low(v);
     }
@@ -285,8 +295,10 @@ __global__ void __launch_bounds__(256, 1) k_lincomb_tc(const __grid_constant__ C
     tc::mbar_init(done_bar, 1);
     tc::fence_mbar_init();
   }
+  pdl_begin();
   if (warp == 0) tc::tmem_alloc(slot, 256);
   tc::fence_before_sync();
+  pdl_wait();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *slot;
@@ -547,7 +559,7 @@ TcGram launch_gram_tc(const Geo &g, const float *X, int nb, const float *uwh, co
   const CUtensorMap mX = rows_map(X, kf, nb, ldf, TM), mUh = rows_map(uwh, kf, na, ldf, nbox), mUl = rows_map(uwl, kf, na, ldf, nbox);
   double *dst = nsplit == 1 ? out : work;
   const size_t stride = nsplit == 1 ? (size_t)0 : (size_t)na * nb;
-  launch("gram", 32, k_gram_tc, dim3(tiles, nsplit, nmc), dim3(kGramThreads), gram_tc_smem(nbox), st, mX, mUh, mUl, g, nb, na, nbox, dst,
+  launch_pdl("gram", 32, (long long)tiles * nsplit * nmc, k_gram_tc, dim3(tiles, nsplit, nmc), dim3(kGramThreads), gram_tc_smem(nbox), st, mX, mUh, mUl, g, nb, na, nbox, dst,
          nb, per, stride, err);
   WDF_CUDA_TRY(cudaGetLastError());
   return {dst, nsplit, stride};
@@ -557,13 +569,13 @@ void launch_lincomb_tc(const Geo &g, float *Y, int ny, const TcGram &S, const do
                        const float *uth, const float *utl, float c0, const float *P, double *part, int *err, cudaStream_t st) {
   if (ny <= 0) return;
   const int kp = tc_rows(na);
-  launch("lincomb", 32, k_tc_coef, dim3((ny + 31) / 32, (kp + 31) / 32), dim3(32, 8), 0, st, S.S, S.nsplit, S.stride, ny, d, na, ny, kp,
+  launch_pdl("lincomb", 32, (long long)((ny + 31) / 32) * (kp / 4), k_tc_coef, dim3((ny + 31) / 32, kp / 4), dim3(32, 8), 0, st, S.S, S.nsplit, S.stride, ny, d, na, ny, kp,
          chi, clo);
   WDF_CUDA_TRY(cudaGetLastError());
   const int ntile = (2 * g.nint + kLinTN - 1) / kLinTN;
   const CUtensorMap mCh = rows_map(chi, kp, ny, kp, TM), mCl = rows_map(clo, kp, ny, kp, TM);
   const CUtensorMap mUh = rows_map(uth, kp, 2 * g.ld, kp, kLinTN), mUl = rows_map(utl, kp, 2 * g.ld, kp, kLinTN);
-  launch("lincomb", 32, k_lincomb_tc, dim3((ny + TM - 1) / TM, ntile), dim3(256), lincomb_tc_smem(), st, mCh, mCl, mUh, mUl, g, Y, ny, kp,
+  launch_pdl("lincomb", 32, (long long)((ny + TM - 1) / TM) * ntile, k_lincomb_tc, dim3((ny + TM - 1) / TM, ntile), dim3(256), lincomb_tc_smem(), st, mCh, mCl, mUh, mUl, g, Y, ny, kp,
          c0, P, part, lincomb_dot_chunks(g), err);
   WDF_CUDA_TRY(cudaGetLastError());
 }

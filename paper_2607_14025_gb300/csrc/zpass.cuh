@@ -31,7 +31,9 @@ __global__ void __launch_bounds__(kThreads) k_zpass_g2r(const cplx<T> *X, int nv
   const int k0 = blockIdx.y * kZCols;
   const int n3 = N3 > 0 ? N3 : g.n3, pitch = n3 + 1, nlines = 2 * kZCols;
   for (int i = threadIdx.x; i < n3; i += blockDim.x) tw[i] = tw3[i];
+  pdl_begin();
   for (int i = threadIdx.x; i < nlines * pitch; i += blockDim.x) sm[i] = mkc<T>(0, 0);
+  pdl_wait();
   __syncthreads();
   const int kend = min(k0 + kZCols, g.K);
   const int e0 = g.col_off[k0], e1 = g.col_off[kend];
@@ -95,6 +97,8 @@ __global__ void __launch_bounds__(kThreads) k_zpass_r2g(const cplx<T> *__restric
   const int k0 = blockIdx.y * kZCols;
   const int n3 = N3 > 0 ? N3 : g.n3, pitch = n3 + 1, nlines = 2 * kZCols;
   for (int i = threadIdx.x; i < n3; i += blockDim.x) tw[i] = tw3[i];
+  pdl_begin();
+  pdl_wait();
   const int kend = min(k0 + kZCols, g.K);
   const int ncol = kend - k0;
   const cplx<T> *in = cb + (size_t)q * n3 * g.ldcb;

@@ -22,7 +22,7 @@ template <typename T, int... Ns> struct ZFastSizes {
   template <int N> static bool g2r_n(const FftCtx<T> &f, const cplx<T> *X, int nvec, cplx<T> *cb, cudaStream_t st) {
     if (f.g.n3 != N) return false;
     const dim3 grid((nvec + 1) / 2, (f.g.K + kZCols - 1) / kZCols);
-    launch("zpass_g2r", bits_of<T>(), k_zpass_g2r<T, false, N>, grid, dim3(kThreads), zfast_smem<T>(N), st, X, nvec, f.g, f.P3, f.tw3,
+    launch_pdl("zpass_g2r", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_g2r<T, false, N>, grid, dim3(kThreads), zfast_smem<T>(N), st, X, nvec, f.g, f.P3, f.tw3,
            cb, PDir<T>());
     WDF_CUDA_TRY(cudaGetLastError());
     return true;
@@ -30,7 +30,7 @@ template <typename T, int... Ns> struct ZFastSizes {
   template <int N> static bool g2r_dir_n(const FftCtx<T> &f, const PDir<T> &d, int nvec, cplx<T> *cb, cudaStream_t st) {
     if (f.g.n3 != N) return false;
     const dim3 grid((nvec + 1) / 2, (f.g.K + kZCols - 1) / kZCols);
-    launch("zpass_g2r", bits_of<T>(), k_zpass_g2r<T, true, N>, grid, dim3(kThreads), zfast_smem<T>(N), st, (const cplx<T> *)d.p, nvec,
+    launch_pdl("zpass_g2r", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_g2r<T, true, N>, grid, dim3(kThreads), zfast_smem<T>(N), st, (const cplx<T> *)d.p, nvec,
            f.g, f.P3, f.tw3, cb, d);
     WDF_CUDA_TRY(cudaGetLastError());
     return true;
@@ -40,11 +40,11 @@ template <typename T, int... Ns> struct ZFastSizes {
     const dim3 grid((nvec + 1) / 2, (f.g.K + kZCols - 1) / kZCols);
     const size_t sm = zfast_smem<T>(N);
     if (epi == EPI_STORE)
-      launch("zpass_r2g", bits_of<T>(), k_zpass_r2g<T, EPI_STORE, N>, grid, dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
+      launch_pdl("zpass_r2g", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_r2g<T, EPI_STORE, N>, grid, dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
     else if (epi == EPI_HSHIFT)
-      launch("zpass_r2g", bits_of<T>(), k_zpass_r2g<T, EPI_HSHIFT, N>, grid, dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
+      launch_pdl("zpass_r2g", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_r2g<T, EPI_HSHIFT, N>, grid, dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
     else
-      launch("zpass_r2g", bits_of<T>(), k_zpass_r2g<T, EPI_DRHO, N>, grid, dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
+      launch_pdl("zpass_r2g", bits_of<T>(), (long long)grid.x * grid.y, k_zpass_r2g<T, EPI_DRHO, N>, grid, dim3(kThreads), sm, st, cb, nvec, f.g, f.P3, f.tw3, ea);
     WDF_CUDA_TRY(cudaGetLastError());
     return true;
   }

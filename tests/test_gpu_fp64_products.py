@@ -1,6 +1,6 @@
 """The FP64 Gram products and linear combinations behind H x, A_v x, W_p x (plain FP64) against
-numpy, at the edges of their 16 x 16 output tiles, of the 4- and 8-vector groups, of the 128-element
-blocks and of the element splits (more than 8 vectors: 8 and fewer take the narrow kernels).
+numpy, at the edges of their 16 x 16 output tiles, of the 1-, 2-, 4- and 8-vector groups, of the
+128-element blocks and of the element splits (Gram products with 8 vectors and fewer: the narrow kernel).
 
 W_p x = v^1/2 sum_a phibar_a lam_a / (1 - lam_a) <phibar_a, v^1/2 x> is one Gram product and one
 combination; both sides sum a few thousand terms in FP64, so they agree to a few hundred ulp:
@@ -49,7 +49,7 @@ def wp_reference(s, lam, phi, x):
 
 
 @pytest.mark.parametrize("n", [24, 45, 64])
-@pytest.mark.parametrize("neig,nvec", [(1, 9), (15, 16), (16, 17), (17, 33), (64, 47), (33, 130), (200, 12)])
+@pytest.mark.parametrize("neig,nvec", [(1, 9), (15, 16), (16, 17), (17, 33), (64, 47), (33, 130), (200, 12), (65, 1), (64, 2), (70, 3), (63, 8)])
 def test_wp_matches_numpy(n, neig, nvec):
     c, s = context(n)
     rng = np.random.default_rng(neig * 1000 + nvec)
