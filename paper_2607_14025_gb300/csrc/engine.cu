@@ -398,12 +398,14 @@ static int apply_operator_cg(wdf_ctx *c, cplx<T> *X, cplx<T> *Y, int n, const do
 // ---------------------------------------------------------------------------------------------
 // preconditioned conjugate gradients on (H - eps_v + alpha P) d = b, one solve per row
 
+// x: the solution; b: the right-hand sides, which an FP32 solve overwrites (its residual starts there)
 template <typename T>
-static void cg_solve(wdf_ctx *c, const cplx<T> *b, cplx<T> *x, int n, int maxiter, std::vector<int> &iters) {
+static void cg_solve(wdf_ctx *c, std::conditional_t<std::is_same<T, float>::value, cplx<T>, const cplx<T>> *b, cplx<T> *x, int n,
+                     int maxiter, std::vector<int> &iters) {
   const Geo &g = c->geo;
   wdf_ctx::Cg &w = Prec<T>::cg(c);
   const size_t vb = sizeof(cplx<T>) * (size_t)n * g.ld;
-  w.r.ensure(vb);
+  if (!std::is_same<T, float>::value) w.r.ensure(vb);
   w.p.ensure(vb);
   w.Ap.ensure(vb);
   const int nch = dot_chunks(g);
@@ -427,7 +429,7 @@ static void cg_solve(wdf_ctx *c, const cplx<T> *b, cplx<T> *x, int n, int maxite
   s.arrived = ii + 2 * n;
   s.nactive = ii + 3 * n;
   s.vidx = c->vidx_dev.as<int>();
-  cplx<T> *r = w.r.as<cplx<T>>(), *p = w.p.as<cplx<T>>(), *Ap = w.Ap.as<cplx<T>>();
+  cplx<T> *r, *p = w.p.as<cplx<T>>(), *Ap = w.Ap.as<cplx<T>>();
   cudaStream_t st = c->st;
   const T *K = c->opt.precond == WDF_PRECOND_TPA ? Prec<T>::kp(c) : nullptr;
   if (c->opt.precond == WDF_PRECOND_LEARNED) {
@@ -445,7 +447,12 @@ static void cg_solve(wdf_ctx *c, const cplx<T> *b, cplx<T> *x, int n, int maxite
   }
 
   WDF_CUDA_TRY(cudaMemsetAsync(x, 0, vb, st));
-  WDF_CUDA_TRY(cudaMemcpyAsync(r, b, vb, cudaMemcpyDeviceToDevice, st));
+  if constexpr (std::is_same<T, float>::value) {
+    r = b;
+  } else {
+    r = w.r.as<cplx<T>>();
+    WDF_CUDA_TRY(cudaMemcpyAsync(r, b, vb, cudaMemcpyDeviceToDevice, st));
+  }
   WDF_CUDA_TRY(cudaMemsetAsync(ii, 0, sizeof(int) * (3 * (size_t)n + 2), st));
   launch_cg_start<T>(g, r, p, K, s, n, nch, st);
   launch_cg_scalars(s, n, nch, maxiter, st);
@@ -615,17 +622,23 @@ void sternheimer_solve(wdf_ctx *c, const cplx<double> *b, cplx<double> *x, const
     WDF_CUDA_TRY(cudaMemcpyAsync(c->krow.p, c->vidx_dev.p, sizeof(int) * n, cudaMemcpyDeviceToDevice, st));
     WDF_CUDA_TRY(cudaMemsetAsync(c->nfb.p, 0, sizeof(int), st));
   }
-  // r = b - A x; A x in FP64, or in double-float (FP64 vectors converted in and out)
-  auto residual = [&]() {
-    if (c->opt.precision == WDF_MIXED_DF) {
+  const bool df = c->opt.precision == WDF_MIXED_DF;
+  // A x in FP64, or in double-float (into dfb; xdf_ready: dfa holds x already)
+  bool xdf_ready = false;
+  auto apply_x = [&]() {
+    if (df) {
       c->dfa.ensure(vb);
       c->dfb.ensure(vb);
-      to_df(c, c->dfa.as<cplx<df64>>(), x, n);
+      if (!xdf_ready) to_df(c, c->dfa.as<cplx<df64>>(), x, n);
       apply_operator<df64>(c, c->dfa.as<cplx<df64>>(), c->dfb.as<cplx<df64>>(), n, c->shift.as<double>(), true);
-      from_df(c, Ax, c->dfb.as<cplx<df64>>(), n);
     } else {
       apply_operator<double>(c, x, Ax, n, c->shift.as<double>(), true);
     }
+  };
+  // r = b - A x with A x left in Ax (calibrate() reads it)
+  auto residual = [&]() {
+    apply_x();
+    if (df) from_df(c, Ax, c->dfb.as<cplx<df64>>(), n);
     WDF_CUDA_TRY(cudaMemcpyAsync(r, b, vb, cudaMemcpyDeviceToDevice, st));
     launch_axpby<double>(g, r, Ax, n, -1.0, 1.0, st);
   };
@@ -660,12 +673,19 @@ void sternheimer_solve(wdf_ctx *c, const cplx<double> *b, cplx<double> *x, const
     epsA *= 16.0;
     if (!std::isfinite(epsA)) epsA = -1.0;
   };
+  // at the top of a refinement step r may be b itself (before the first correction: <r, r> = <b, b>, no copy),
+  // or k_residual_end has left its FP32 copy in rwork and the partial sums of <r, r> in cg64.part1
+  enum { kNothing, kIsRhs, kSummed } known = kNothing;
+  const cplx<double> *rcur = r;  // the residual: b itself before the first correction
+  bool x_zero = true;
   if (learned && c->opt.warm_start) {  // x0 = o1 K b from the model, then its residual
     launch_first_iterate(g, x, b, c->mlw64.as<double>(), c->vidx_dev.as<int>(), n, st);
+    x_zero = false;
     residual();
   } else {
     WDF_CUDA_TRY(cudaMemsetAsync(x, 0, vb, st));
-    WDF_CUDA_TRY(cudaMemcpyAsync(r, b, vb, cudaMemcpyDeviceToDevice, st));
+    known = kIsRhs;
+    rcur = b;
   }
   const double tol = c->opt.cg_tol;
   const int maxref = mixed ? 12 : 6;
@@ -676,8 +696,17 @@ void sternheimer_solve(wdf_ctx *c, const cplx<double> *b, cplx<double> *x, const
   ss.refinements = 0;
   const bool trace = std::getenv("WDF_TRACE") != nullptr;
   for (int ref = 0; ref <= maxref; ++ref) {
-    dots<double>(c, r, r, n, nrm);
-    rr = to_host(c, nrm, n);
+    if (known == kIsRhs) {
+      rr = bb;
+    } else {
+      if (known == kSummed) {
+        launch("sum_chunks", 0, k_sum_chunks, dim3((n + 127) / 128), dim3(128), 0, st, c->cg64.part1.as<double>(), n, dot_chunks(g), nrm);
+        WDF_CUDA_TRY(cudaGetLastError());
+      } else {
+        dots<double>(c, r, r, n, nrm);
+      }
+      rr = to_host(c, nrm, n);
+    }
     int nact = 0, nunconv = 0;
     double worst = 0.0;
     for (int s = 0; s < n; ++s) {
@@ -719,11 +748,18 @@ void sternheimer_solve(wdf_ctx *c, const cplx<double> *b, cplx<double> *x, const
       w.x.ensure(sizeof(cplx<float>) * (size_t)n * g.ld);
       c->rwork.ensure(sizeof(cplx<float>) * (size_t)n * g.ld);
       cplx<float> *r32 = c->rwork.as<cplx<float>>(), *d32 = w.x.as<cplx<float>>();
-      launch_convert<double, float>(g, (float *)r32, (const double *)r, 2 * (size_t)n * g.ld, st);
+      if (known != kSummed) launch_convert<double, float>(g, (float *)r32, (const double *)rcur, 2 * (size_t)n * g.ld, st);
       cg_solve<float>(c, r32, d32, n, budget, it);
-      // x += d ; reuse Ax as FP64 staging of d
-      launch_convert<float, double>(g, (double *)Ax, (const float *)d32, 2 * (size_t)n * g.ld, st);
-      launch_axpby<double>(g, x, Ax, n, 1.0, 1.0, st);
+      if (may_update) {  // x += d with Ax as FP64 staging of d
+        if (x_zero && rcur != r) WDF_CUDA_TRY(cudaMemcpyAsync(r, b, vb, cudaMemcpyDeviceToDevice, st));
+        launch_convert<float, double>(g, (double *)Ax, (const float *)d32, 2 * (size_t)n * g.ld, st);
+        launch_axpby<double>(g, x, Ax, n, 1.0, 1.0, st);
+      } else {
+        if (df) c->dfa.ensure(vb);
+        launch_add_correction(x, d32, df ? c->dfa.as<cplx<df64>>() : nullptr, (size_t)n * g.ld, x_zero, st);
+        xdf_ready = df;
+      }
+      x_zero = false;
       if (epsA >= 0.0 && may_update) {  // r - A_32 d when every bound stays small
         dots<double>(c, Ax, Ax, n, nrm + n);
         const std::vector<double> dd = to_host(c, nrm + n, n);
@@ -744,13 +780,25 @@ void sternheimer_solve(wdf_ctx *c, const cplx<double> *b, cplx<double> *x, const
       auto &w = c->cg64;
       w.x.ensure(vb);
       cplx<double> *d = w.x.as<cplx<double>>();
-      cg_solve<double>(c, r, d, n, budget, it);
+      cg_solve<double>(c, rcur, d, n, budget, it);
       launch_axpby<double>(g, x, d, n, 1.0, 1.0, st);
     }
+    rcur = r;
+    known = kNothing;
     for (int s = 0; s < n; ++s) iters_total[s] += it[s];
     if (trace) fprintf(stderr, "[wdf] refinement %d: %s residual (eps_A %.3e)\n", ref, updated ? "updated" : "full", epsA);
     if (!updated) {
-      residual();
+      if (mixed && !may_update) {  // A x, then r, its FP32 copy and <r, r> in one pass
+        apply_x();
+        const int nch = dot_chunks(g);
+        c->cg64.part1.ensure(sizeof(double) * (size_t)n * nch);
+        c->rwork.ensure(sizeof(cplx<float>) * (size_t)n * g.ld);
+        if (df) launch_residual_end<df64>(g, b, c->dfb.as<cplx<df64>>(), r, c->rwork.as<cplx<float>>(), n, c->cg64.part1.as<double>(), nch, st);
+        else launch_residual_end<double>(g, b, Ax, r, c->rwork.as<cplx<float>>(), n, c->cg64.part1.as<double>(), nch, st);
+        known = kSummed;
+      } else {
+        residual();
+      }
       std::fill(bnd.begin(), bnd.end(), 0.0);
       if (may_update && epsA < 0.0) calibrate();
     }

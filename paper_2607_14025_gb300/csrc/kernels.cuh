@@ -152,6 +152,12 @@ template <typename T>
 void launch_dot_partial(const Geo &g, const cplx<T> *A, const cplx<T> *B, int nvec, double *part, int nchunk,
                         cudaStream_t st);
 int dot_chunks(const Geo &g);
+// r = b - Ax (Ax FP64 or double-float), r32 = r in FP32, partial <r, r> as launch_dot_partial
+template <typename S>
+void launch_residual_end(const Geo &g, const cplx<double> *b, const cplx<S> *Ax, cplx<double> *r, cplx<float> *r32, int nvec, double *part,
+                         int nchunk, cudaStream_t st);
+// x += d (x = d when first), xdf = x in double-float when not null; count complex elements
+void launch_add_correction(cplx<double> *x, const cplx<float> *d, cplx<df64> *xdf, size_t count, bool first, cudaStream_t st);
 // part[s * nchunk + c] = sum over chunk c of w_e |A_s[e] - B_s[e]|^2 (A FP64, B FP32)
 void launch_diff_partial(const Geo &g, const cplx<double> *A, const cplx<float> *B, int nvec, double *part, int nchunk, cudaStream_t st);
 
