@@ -105,27 +105,28 @@ const double *stage_in(wdf_ctx *c, DBuf &buf, const double *src, size_t ndouble,
   return buf.as<double>();
 }
 
-// copy internal FP64 vectors out to the caller in external layout
-void write_out(wdf_ctx *c, DBuf &stage, const cplx<double> *in, int n, double *dst, int mem) {
+// copy internal vectors (FP64 or double-float) out to the caller in external layout
+template <typename S> void write_out(wdf_ctx *c, DBuf &stage, const cplx<S> *in, int n, double *dst, int mem) {
   const size_t nd = 2 * (size_t)n * c->npw_h;
   double *target = dst;
   if (mem == WDF_MEM_HOST) {
     stage.ensure(nd * sizeof(double));
     target = stage.as<double>();
   }
-  launch_int_to_ext(in, n, c->geo.ld, c->npw_h, c->t_emap.as<int>(), c->t_econj.as<int>(), target, c->st);
+  launch_int_to_ext<S>(in, n, c->geo.ld, c->npw_h, c->t_emap.as<int>(), c->t_econj.as<int>(), target, c->st);
   if (mem == WDF_MEM_HOST) WDF_CUDA_TRY(cudaMemcpyAsync(dst, target, nd * sizeof(double), cudaMemcpyDeviceToHost, c->st));
 }
 
-// external -> internal FP64 (into buf), optional per-element scale
-cplx<double> *read_in(wdf_ctx *c, DBuf &stage, DBuf &buf, const double *src, int n, int mem, int extra_rows = 0) {
+// external -> internal (into buf), FP64 or double-float
+template <typename S = double>
+cplx<S> *read_in(wdf_ctx *c, DBuf &stage, DBuf &buf, const double *src, int n, int mem, int extra_rows = 0) {
   const double *d = stage_in(c, stage, src, 2 * (size_t)n * c->npw_h, mem);
-  const size_t bytes = sizeof(cplx<double>) * (size_t)(n + extra_rows) * c->geo.ld;
+  const size_t bytes = sizeof(cplx<S>) * (size_t)(n + extra_rows) * c->geo.ld;
   buf.ensure(bytes);
   WDF_CUDA_TRY(cudaMemsetAsync(buf.p, 0, bytes, c->st));
-  launch_ext_to_int(d, n, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr,
-                    buf.as<cplx<double>>(), c->geo.ld, c->st);
-  return buf.as<cplx<double>>();
+  launch_ext_to_int<S>(d, n, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr,
+                    buf.as<cplx<S>>(), c->geo.ld, c->st);
+  return buf.as<cplx<S>>();
 }
 
 template <class T> void upload(wdf_ctx *c, DBuf &b, const std::vector<T> &h) {
@@ -282,7 +283,7 @@ void setup_body(wdf_ctx *c, const wdf_system *sys) {
   WDF_CUDA_TRY(cudaMemsetAsync(c->U64.p, 0, sizeof(cplx<double>) * (size_t)M * g.ld, c->st));
   if (c->nproj > 0) {
     const double *d = stage_in(c, c->ext_in, sys->beta, 2 * (size_t)c->nproj * c->npw_h, sys->mem);
-    launch_ext_to_int(d, c->nproj, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr,
+    launch_ext_to_int<double>(d, c->nproj, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr,
                       c->U64.as<cplx<double>>(), g.ld, c->st);
   }
   c->lrd.ensure(sizeof(double) * M);
@@ -303,7 +304,7 @@ void setup_body(wdf_ctx *c, const wdf_system *sys) {
   int status = WDF_OK;
   if (sys->psi) {
     const double *d = stage_in(c, c->ext_in, sys->psi, 2 * (size_t)c->nocc * c->npw_h, sys->mem);
-    launch_ext_to_int(d, c->nocc, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr,
+    launch_ext_to_int<double>(d, c->nocc, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr,
                       c->U64.as<cplx<double>>() + (size_t)c->nproj * g.ld, g.ld, c->st);
     c->eps.assign(sys->eps, sys->eps + c->nocc);
     for (double e : c->eps)
@@ -351,7 +352,7 @@ struct UserOp : DavOp {
     const size_t nd = 2 * (size_t)n * c->npw_h;
     c->uop_in.ensure(nd * sizeof(double));
     c->uop_out.ensure(nd * sizeof(double));
-    launch_int_to_ext(X, n, c->geo.ld, c->npw_h, c->t_emap.as<int>(), c->t_econj.as<int>(), c->uop_in.as<double>(), c->st);
+    launch_int_to_ext<double>(X, n, c->geo.ld, c->npw_h, c->t_emap.as<int>(), c->t_econj.as<int>(), c->uop_in.as<double>(), c->st);
     WDF_CUDA_TRY(cudaMemsetAsync(c->uop_out.p, 0, nd * sizeof(double), c->st));
     WDF_CUDA_TRY(cudaStreamSynchronize(c->st));  // the callback may work on any stream
     const int rc = fn(user, n, c->uop_in.as<double>(), c->uop_out.as<double>());
@@ -359,7 +360,7 @@ struct UserOp : DavOp {
     ++calls;
     const size_t bytes = sizeof(cplx<double>) * (size_t)n * c->geo.ld;
     WDF_CUDA_TRY(cudaMemsetAsync(Y, 0, bytes, c->st));
-    launch_ext_to_int(c->uop_out.as<double>(), n, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr, Y,
+    launch_ext_to_int<double>(c->uop_out.as<double>(), n, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr, Y,
                       c->geo.ld, c->st);
   }
 };
@@ -472,7 +473,7 @@ int wdf_get_orbitals(wdf_ctx *c, double *eps, double *psi, int mem) {
     check_mem(mem);
     memcpy(eps, c->eps.data(), sizeof(double) * c->nocc);
     if (psi) {
-      write_out(c, c->ext_out, c->U64.as<cplx<double>>() + (size_t)c->nproj * c->geo.ld, c->nocc, psi, mem);
+      write_out<double>(c, c->ext_out, c->U64.as<cplx<double>>() + (size_t)c->nproj * c->geo.ld, c->nocc, psi, mem);
       WDF_CUDA_TRY(cudaStreamSynchronize(c->st));
     }
     return WDF_OK;
@@ -488,7 +489,7 @@ int wdf_apply_hamiltonian(wdf_ctx *c, int nvec, const double *in, double *out, i
     cplx<double> *X = read_in(c, c->ext_in, c->xpert, in, nvec, mem);
     c->outi.ensure(sizeof(cplx<double>) * (size_t)nvec * c->geo.ld);
     apply_operator<double>(c, X, c->outi.as<cplx<double>>(), nvec, nullptr, false);
-    write_out(c, c->ext_out, c->outi.as<cplx<double>>(), nvec, out, mem);
+    write_out<double>(c, c->ext_out, c->outi.as<cplx<double>>(), nvec, out, mem);
     WDF_CUDA_TRY(cudaStreamSynchronize(c->st));
     return WDF_OK;
   });
@@ -508,11 +509,16 @@ int wdf_apply_sternheimer_operator(wdf_ctx *c, int nvec, const int32_t *vidx, co
     for (int s = 0; s < nvec; ++s)
       if (vidx[s] < 0 || vidx[s] >= c->nocc) throw ApiFailure(WDF_EINVAL, "vidx out of range");
     if (nvec == 0) return WDF_OK;
-    cplx<double> *X = read_in(c, c->ext_in, c->xpert, in, nvec, mem);
-    c->outi.ensure(sizeof(cplx<double>) * (size_t)nvec * c->geo.ld);
-    std::vector<int> v(vidx, vidx + nvec);
-    apply_sternheimer_operator(c, X, c->outi.as<cplx<double>>(), v.data(), nvec);
-    write_out(c, c->ext_out, c->outi.as<cplx<double>>(), nvec, out, mem);
+    const std::vector<int> v(vidx, vidx + nvec);
+    auto run = [&](auto zero) {  // in the precision of the residuals
+      typedef decltype(zero) S;
+      const cplx<S> *X = read_in<S>(c, c->ext_in, c->xpert, in, nvec, mem);
+      c->outi.ensure(sizeof(cplx<S>) * (size_t)nvec * c->geo.ld);
+      apply_sternheimer_operator<S>(c, X, c->outi.as<cplx<S>>(), v.data(), nvec);
+      write_out<S>(c, c->ext_out, c->outi.as<cplx<S>>(), nvec, out, mem);
+    };
+    if (c->opt.precision == WDF_MIXED_DF) run(df64());
+    else run(0.0);
     WDF_CUDA_TRY(cudaStreamSynchronize(c->st));
     return WDF_OK;
   });
@@ -532,7 +538,7 @@ int wdf_sternheimer(wdf_ctx *c, int nsolve, const int32_t *vidx, const double *r
       c->rx.ensure(sizeof(cplx<double>) * (size_t)nsolve * c->geo.ld);
       std::vector<int> v(vidx, vidx + nsolve);
       sternheimer_solve(c, B, c->rx.as<cplx<double>>(), v.data(), nsolve, ss);
-      write_out(c, c->ext_out, c->rx.as<cplx<double>>(), nsolve, x, mem);
+      write_out<double>(c, c->ext_out, c->rx.as<cplx<double>>(), nsolve, x, mem);
       WDF_CUDA_TRY(cudaStreamSynchronize(c->st));
     }
     fill_stats(st, ss, nsolve, 0, tm.ms());
@@ -553,8 +559,8 @@ int wdf_apply_chi0(wdf_ctx *c, int npert, const double *phi, double *out, double
       c->outi.ensure(sizeof(cplx<double>) * (size_t)np2 * c->geo.ld);
       c->drhoi.ensure(sizeof(cplx<double>) * (size_t)np2 * c->geo.ld);
       chi0_apply_internal(c, P, npert, c->outi.as<cplx<double>>(), c->drhoi.as<cplx<double>>(), ss);
-      write_out(c, c->ext_out, c->outi.as<cplx<double>>(), npert, out, mem);
-      if (drho) write_out(c, c->ext_out2, c->drhoi.as<cplx<double>>(), npert, drho, mem);
+      write_out<double>(c, c->ext_out, c->outi.as<cplx<double>>(), npert, out, mem);
+      if (drho) write_out<double>(c, c->ext_out2, c->drhoi.as<cplx<double>>(), npert, drho, mem);
       WDF_CUDA_TRY(cudaStreamSynchronize(c->st));
     }
     fill_stats(st, ss, (long long)npert * c->nocc, npert, tm.ms());
@@ -579,7 +585,7 @@ int wdf_apply_wp(wdf_ctx *c, int neig, const double *lambda, const double *phiba
     WDF_CUDA_TRY(cudaMemcpyAsync(c->wp_coef.p, coef.data(), sizeof(double) * neig, cudaMemcpyHostToDevice, c->st));
     c->wp_y.ensure(sizeof(cplx<double>) * (size_t)nvec * c->geo.ld);
     wp_apply_internal(c, P, c->wp_coef.as<double>(), neig, X, nvec, c->wp_y.as<cplx<double>>());
-    write_out(c, c->ext_out, c->wp_y.as<cplx<double>>(), nvec, out, mem);
+    write_out<double>(c, c->ext_out, c->wp_y.as<cplx<double>>(), nvec, out, mem);
     WDF_CUDA_TRY(cudaStreamSynchronize(c->st));
     return WDF_OK;
   });
@@ -665,7 +671,7 @@ int wdf_pdep_davidson(wdf_ctx *c, int neig, int nbasis_max, int maxiter, double 
     Chi0Op op(c);
     DavResult r = davidson(c, op, G0, nguess, neig, neig, nbmax, maxiter, tol, true);
     for (int a = 0; a < neig; ++a) lambda[a] = r.lam[a];
-    write_out(c, c->ext_out, c->dv_X.as<cplx<double>>(), neig, phibar, mem);
+    write_out<double>(c, c->ext_out, c->dv_X.as<cplx<double>>(), neig, phibar, mem);
     WDF_CUDA_TRY(cudaStreamSynchronize(c->st));
     op.agg.converged = op.agg.converged && r.converged;
     fill_stats(st, op.agg, op.nsolve, r.napply, tm.ms());
@@ -693,7 +699,7 @@ int wdf_davidson(wdf_ctx *c, wdf_operator_fn apply, void *user, int neig, int nb
     UserOp op(c, apply, user);
     DavResult r = davidson(c, op, G0, nguess, neig, neig, nbmax, maxiter, tol, zero_g0 != 0);
     for (int a = 0; a < neig; ++a) lambda[a] = r.lam[a];
-    write_out(c, c->ext_out, c->dv_X.as<cplx<double>>(), neig, vec, mem);
+    write_out<double>(c, c->ext_out, c->dv_X.as<cplx<double>>(), neig, vec, mem);
     WDF_CUDA_TRY(cudaStreamSynchronize(c->st));
     SolveStats none;
     none.converged = r.converged;

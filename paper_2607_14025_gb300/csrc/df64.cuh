@@ -16,6 +16,8 @@
 
 #include <cuda_runtime.h>
 
+#include "convert_bits.cuh"
+
 namespace wdf {
 
 struct df64 {
@@ -29,6 +31,13 @@ struct df64 {
   __host__ __device__ explicit operator double() const { return (double)hi + (double)lo; }
   __host__ __device__ explicit operator float() const { return hi + lo; }
 };
+
+// the casts of passes over whole vectors: one FP64 operation each way, the conversions on the integer units
+__device__ __forceinline__ df64 split_double(double d) {
+  const float h = narrow(d);
+  return df64(h, narrow(d - widen(h)));
+}
+__device__ __forceinline__ double join_double(df64 v) { return widen(v.hi) + widen(v.lo); }
 
 // The error-free steps use the round-to-nearest intrinsics, which the compiler never contracts
 // into fused multiply-adds (a contraction would break the exactness the transformations rely on).

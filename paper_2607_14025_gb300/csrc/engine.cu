@@ -565,7 +565,8 @@ static void cg_solve(wdf_ctx *c, std::conditional_t<std::is_same<T, float>::valu
   WDF_CUDA_TRY(cudaStreamSynchronize(st));
 }
 
-void apply_sternheimer_operator(wdf_ctx *c, const cplx<double> *X, cplx<double> *Y, const int *vidx_host, int n) {
+template <typename S>
+void apply_sternheimer_operator(wdf_ctx *c, const cplx<S> *X, cplx<S> *Y, const int *vidx_host, int n) {
   if (n <= 0) return;
   const Geo &g = c->geo;
   cudaStream_t st = c->st;
@@ -575,21 +576,14 @@ void apply_sternheimer_operator(wdf_ctx *c, const cplx<double> *X, cplx<double> 
   launch("gather_shift", 0, k_gather_shift, dim3((n + 127) / 128), dim3(128), 0, st, c->vidx_dev.as<int>(), c->eps_dev.as<double>(),
          c->shift.as<double>(), n);
   WDF_CUDA_TRY(cudaGetLastError());
-  if (c->opt.precision == WDF_MIXED_DF) {
-    const size_t vb = sizeof(cplx<double>) * (size_t)n * g.ld;
-    c->dfa.ensure(vb);
-    c->dfb.ensure(vb);
-    to_df(c, c->dfa.as<cplx<df64>>(), X, n);
-    apply_operator<df64>(c, c->dfa.as<cplx<df64>>(), c->dfb.as<cplx<df64>>(), n, c->shift.as<double>(), true);
-    from_df(c, Y, c->dfb.as<cplx<df64>>(), n);
-  } else {
-    apply_operator<double>(c, X, Y, n, c->shift.as<double>(), true);
-  }
+  apply_operator<S>(c, X, Y, n, c->shift.as<double>(), true);
   int terr = 0;
   WDF_CUDA_TRY(cudaMemcpyAsync(&terr, c->tcerr.p, sizeof(int), cudaMemcpyDeviceToHost, st));
   WDF_CUDA_TRY(cudaStreamSynchronize(st));
   if (terr) throw ApiFailure(WDF_ETIMEOUT, "a kernel gave up waiting for its MMAs or bulk copies");
 }
+template void apply_sternheimer_operator<double>(wdf_ctx *, const cplx<double> *, cplx<double> *, const int *, int);
+template void apply_sternheimer_operator<df64>(wdf_ctx *, const cplx<df64> *, cplx<df64> *, const int *, int);
 
 // FP64 outer loop: r = b - A x in FP64, inner solve A d = r (FP64 or FP32), x += d.
 void sternheimer_solve(wdf_ctx *c, const cplx<double> *b, cplx<double> *x, const int *vidx_host, int n, SolveStats &ss) {

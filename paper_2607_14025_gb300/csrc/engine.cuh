@@ -133,7 +133,7 @@ template <typename T>
 void apply_operator(wdf_ctx *c, const cplx<T> *X, cplx<T> *Y, int n, const double *shift, bool with_alpha);
 // A_v x = (H - eps_v + alpha P) x in the precision of the residuals (FP64, or double-float for
 // WDF_MIXED_DF); vidx_host: [n] orbital of each vector
-void apply_sternheimer_operator(wdf_ctx *c, const cplx<double> *X, cplx<double> *Y, const int *vidx_host, int n);
+template <typename S> void apply_sternheimer_operator(wdf_ctx *c, const cplx<S> *X, cplx<S> *Y, const int *vidx_host, int n);
 
 struct SolveStats {
   long long iters = 0;

@@ -736,10 +736,22 @@ __global__ void __launch_bounds__(256) k_diff_partial(Geo g, const cplx<double> 
   if (threadIdx.x == 0) part[(size_t)s * nchunk + c] = v;
 }
 
+// casts with the conversions on the integer units (convert_bits.cuh)
+template <typename To> __device__ __forceinline__ To cast(double v);
+template <> __device__ __forceinline__ double cast<double>(double v) { return v; }
+template <> __device__ __forceinline__ float cast<float>(double v) { return narrow(v); }
+template <> __device__ __forceinline__ df64 cast<df64>(double v) { return split_double(v); }
+template <typename To> __device__ __forceinline__ To cast(float v);
+template <> __device__ __forceinline__ double cast<double>(float v) { return widen(v); }
+template <typename To> __device__ __forceinline__ To cast(df64 v);
+template <> __device__ __forceinline__ double cast<double>(df64 v) { return join_double(v); }
+
 // The end of a residual in one pass: r = b - Ax (Ax FP64 or double-float), its FP32 copy for the inner
 // iterations and the partial sums of <r, r> in the chunks of k_dot_partial. As a conversion, a copy of b,
 // an update, a dot product and a conversion this moved 168 bytes per element; here 72. With k_add_correction
 // a chi0 application of 2,048 solves on 64^3 went from 87.2 to 86.1 ms, of 1,536 on 96^3 from 274 to 270 ms.
+// Bound by HBM and, nearly as much, by the FP64 pipe: 7 operations per element with the conversions on the
+// integer units (0.51 ms for 1,536 rows of 23,168), 13 with the conversion instructions (0.90 ms).
 template <typename S>
 __global__ void __launch_bounds__(256) k_residual_end(Geo g, const cplx<double> *__restrict__ b, const cplx<S> *__restrict__ Ax,
                                                      cplx<double> *__restrict__ r, cplx<float> *__restrict__ r32, double *__restrict__ part,
@@ -754,10 +766,10 @@ __global__ void __launch_bounds__(256) k_residual_end(Geo g, const cplx<double> 
     if (e < e1) {
       const cplx<S> a = Ax[o + e];
       const cplx<double> bv = b[o + e];
-      rv = mkc<double>(bv.x - (double)a.x, bv.y - (double)a.y);
+      rv = mkc<double>(bv.x - cast<double>(a.x), bv.y - cast<double>(a.y));
     }
     r[o + e] = rv;
-    r32[o + e] = mkc<float>((float)rv.x, (float)rv.y);
+    r32[o + e] = mkc<float>(narrow(rv.x), narrow(rv.y));
     if (e < e1) v += wgt(e, g.len0) * dre<double>(rv, rv);
   }
   v = block_sum(v);
@@ -776,16 +788,16 @@ template void launch_residual_end<df64>(const Geo &, const cplx<double> *, const
                                         int, cudaStream_t);
 
 // x += d for an FP32 correction d (x = d when first), with the double-float copy of the new x for the
-// residual when xdf is given
+// residual when xdf is given; 0.35 ms for 1,536 rows of 23,168, 0.78 with the conversion instructions
 __global__ void __launch_bounds__(256) k_add_correction(cplx<double> *__restrict__ x, const cplx<float> *__restrict__ d,
                                                        cplx<df64> *__restrict__ xdf, size_t count, bool first) {
 #pragma unroll 4
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < count; t += (size_t)gridDim.x * blockDim.x) {
     const cplx<float> dv = d[t];
     const cplx<double> o = first ? mkc<double>(0.0, 0.0) : x[t];
-    const cplx<double> xv = mkc<double>(o.x + (double)dv.x, o.y + (double)dv.y);
+    const cplx<double> xv = mkc<double>(o.x + widen(dv.x), o.y + widen(dv.y));
     x[t] = xv;
-    if (xdf) xdf[t] = mkc<df64>(df64(xv.x), df64(xv.y));
+    if (xdf) xdf[t] = mkc<df64>(split_double(xv.x), split_double(xv.y));
   }
 }
 void launch_add_correction(cplx<double> *x, const cplx<float> *d, cplx<df64> *xdf, size_t count, bool first, cudaStream_t st) {
@@ -1087,9 +1099,19 @@ template <typename T> void launch_scale_rows(const Geo &g, cplx<T> *y, const dou
   WDF_CUDA_TRY(cudaGetLastError());
 }
 
+// 4 values of a thread in flight; y and x may be any arrays of the element types
 template <typename Tin, typename Tout>
-__global__ void k_convert(Tout *__restrict__ y, const Tin *__restrict__ x, size_t count) {
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < count; t += (size_t)gridDim.x * blockDim.x) y[t] = (Tout)x[t];
+__global__ void __launch_bounds__(256) k_convert(Tout *__restrict__ y, const Tin *__restrict__ x, size_t count) {
+  const size_t step = (size_t)gridDim.x * blockDim.x;
+  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < count; t += 4 * step) {
+    Tin v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (t + u * step < count) v[u] = x[t + u * step];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (t + u * step < count) y[t + u * step] = cast<Tout>(v[u]);
+  }
 }
 // the orbital sum of the density response on the grid: acc = sum_v psi_v(r) G2R(dpsi_v pair)(r),
 // the orbitals in ascending order (the same order as the in-plane sums)
@@ -1125,51 +1147,78 @@ template void launch_fill<df64>(df64 *, size_t, double, cudaStream_t);
 
 template <typename Tin, typename Tout> void launch_convert(const Geo &, Tout *y, const Tin *x, size_t count, cudaStream_t st) {
   if (count == 0) return;
-  launch("convert", bits_of<Tout>(), k_convert<Tin, Tout>, dim3((int)std::min<size_t>(8192, (count + 255) / 256)), dim3(256), 0, st, y, x, count);
+  launch("convert", bits_of<Tout>(), k_convert<Tin, Tout>, dim3((int)std::min<size_t>(8 * 152, (count + 255) / 256)), dim3(256), 0, st, y, x, count);
   WDF_CUDA_TRY(cudaGetLastError());
 }
 
-__global__ void k_ext_to_int(const double *__restrict__ ext, int n, int npw_h, const int *__restrict__ emap,
+// External half-sphere vectors -> the internal layout, in FP64 or directly in double-float. A block takes
+// 256 coefficients of one row after the other (their map entries stay in registers). 512 rows of 23,168
+// take 189 us in double-float; with 64-bit divisions per coefficient and the split as a pass of its own
+// 142 + 172 us.
+template <typename S>
+__global__ void __launch_bounds__(256) k_ext_to_int(const double *__restrict__ ext, int n, int npw_h, const int *__restrict__ emap,
                              const int *__restrict__ emap2, const int *__restrict__ econj, const double *__restrict__ scale,
-                             cplx<double> *__restrict__ out, int ld) {
-  const size_t tot = (size_t)n * npw_h;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < tot; t += (size_t)gridDim.x * blockDim.x) {
-    const int s = (int)(t / npw_h), i = (int)(t % npw_h);
-    double re = ext[2 * t], im = ext[2 * t + 1];
-    const int e = emap[i];
-    if (i == 0) im = 0.0;  // G = 0 coefficient of a real function is real
-    if (econj[i]) im = -im;
-    const double sc = scale ? scale[e] : 1.0;
-    out[(size_t)s * ld + e] = mkc<double>(sc * re, sc * im);
-    const int e2 = emap2[i];
-    if (e2 >= 0) out[(size_t)s * ld + e2] = mkc<double>(sc * re, -sc * im);
+                             cplx<S> *__restrict__ out, int ld) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= npw_h) return;
+  const int e = emap[i], e2 = emap2[i];
+  const bool conj = econj[i] != 0;
+  const double sc = scale ? scale[e] : 1.0;
+#pragma unroll 4
+  for (int s = blockIdx.y; s < n; s += gridDim.y) {
+    const double *v = ext + 2 * ((size_t)s * npw_h + i);
+    double re = v[0], im = i == 0 ? 0.0 : v[1];  // G = 0 coefficient of a real function is real
+    if (conj) im = -im;
+    if (scale) {
+      re *= sc;
+      im *= sc;
+    }
+    const S x = cast<S>(re), y = cast<S>(im);
+    out[(size_t)s * ld + e] = mkc<S>(x, y);
+    if (e2 >= 0) out[(size_t)s * ld + e2] = mkc<S>(x, -y);
   }
 }
+static dim3 ext_grid(int n, int npw_h) {
+  const int nb = (npw_h + 255) / 256;
+  return dim3(nb, std::min(n, std::max(1, 16 * 152 / nb)));
+}
+template <typename S>
 void launch_ext_to_int(const double *ext, int n, int npw_h, const int *emap, const int *emap2, const int *econj,
-                       const double *scale_int, cplx<double> *out, int ld, cudaStream_t st) {
+                       const double *scale_int, cplx<S> *out, int ld, cudaStream_t st) {
   if (n <= 0) return;
-  const size_t tot = (size_t)n * npw_h;
-  launch("ext_to_int", 0, k_ext_to_int, dim3((int)std::min<size_t>(8192, (tot + 255) / 256)), dim3(256), 0, st, ext, n, npw_h, emap, emap2, econj, scale_int, out, ld);
+  launch("ext_to_int", 0, k_ext_to_int<S>, ext_grid(n, npw_h), dim3(256), 0, st, ext, n, npw_h, emap, emap2, econj, scale_int, out, ld);
   WDF_CUDA_TRY(cudaGetLastError());
 }
+template void launch_ext_to_int<double>(const double *, int, int, const int *, const int *, const int *, const double *, cplx<double> *, int,
+                                        cudaStream_t);
+template void launch_ext_to_int<df64>(const double *, int, int, const int *, const int *, const int *, const double *, cplx<df64> *, int,
+                                      cudaStream_t);
 
-__global__ void k_int_to_ext(const cplx<double> *__restrict__ in, int n, int ld, int npw_h, const int *__restrict__ emap,
+template <typename S>
+__global__ void __launch_bounds__(256) k_int_to_ext(const cplx<S> *__restrict__ in, int n, int ld, int npw_h, const int *__restrict__ emap,
                              const int *__restrict__ econj, double *__restrict__ ext) {
-  const size_t tot = (size_t)n * npw_h;
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < tot; t += (size_t)gridDim.x * blockDim.x) {
-    const int s = (int)(t / npw_h), i = (int)(t % npw_h);
-    const cplx<double> v = in[(size_t)s * ld + emap[i]];
-    ext[2 * t] = v.x;
-    ext[2 * t + 1] = (i == 0) ? 0.0 : (econj[i] ? -v.y : v.y);
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= npw_h) return;
+  const int e = emap[i];
+  const bool conj = econj[i] != 0;
+#pragma unroll 4
+  for (int s = blockIdx.y; s < n; s += gridDim.y) {
+    const cplx<S> v = in[(size_t)s * ld + e];
+    const double re = cast<double>(v.x), im = cast<double>(v.y);
+    double *o = ext + 2 * ((size_t)s * npw_h + i);
+    o[0] = re;
+    o[1] = i == 0 ? 0.0 : conj ? -im : im;
   }
 }
-void launch_int_to_ext(const cplx<double> *in, int n, int ld, int npw_h, const int *emap, const int *econj, double *ext,
+template <typename S>
+void launch_int_to_ext(const cplx<S> *in, int n, int ld, int npw_h, const int *emap, const int *econj, double *ext,
                        cudaStream_t st) {
   if (n <= 0) return;
-  const size_t tot = (size_t)n * npw_h;
-  launch("int_to_ext", 0, k_int_to_ext, dim3((int)std::min<size_t>(8192, (tot + 255) / 256)), dim3(256), 0, st, in, n, ld, npw_h, emap, econj, ext);
+  launch("int_to_ext", 0, k_int_to_ext<S>, ext_grid(n, npw_h), dim3(256), 0, st, in, n, ld, npw_h, emap, econj, ext);
   WDF_CUDA_TRY(cudaGetLastError());
 }
+template void launch_int_to_ext<double>(const cplx<double> *, int, int, int, const int *, const int *, double *, cudaStream_t);
+template void launch_int_to_ext<df64>(const cplx<df64> *, int, int, int, const int *, const int *, double *, cudaStream_t);
 
 __global__ void k_ritz_residual(Geo g, cplx<double> *__restrict__ R, const cplx<double> *__restrict__ AX,
                                 const cplx<double> *__restrict__ X, const double *__restrict__ theta, int n) {

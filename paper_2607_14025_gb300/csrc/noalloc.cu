@@ -97,7 +97,7 @@ extern "C" int wdf_apply_hamiltonian_noalloc(wdf_ctx *c, int nvec, const double 
     // the padding of X and the shifts must be zero; everything else is written before it is read
     WDF_CUDA_TRY(cudaMemsetAsync(X, 0, bx, st));
     WDF_CUDA_TRY(cudaMemsetAsync(zs, 0, bz, st));
-    launch_ext_to_int(in, nvec, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr, X, g.ld, st);
+    launch_ext_to_int<double>(in, nvec, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr, X, g.ld, st);
     // H x = 1/2|G|^2 x + fft_n(V_loc ifft(x)) + sum_j beta_j D_j <beta_j, x>
     launch_zpass_g2r<double>(c->f64, X, nvec, cb, st);
     PlaneArgs<double> pa;
@@ -114,7 +114,7 @@ extern "C" int wdf_apply_hamiltonian_noalloc(wdf_ctx *c, int nvec, const double 
       launch_gram<double>(g, c->U64.as<cplx<double>>(), M, X, nvec, S, nvec, gw, bgw / sizeof(double), st);
       launch_lincomb<double>(g, Y, nvec, c->U64.as<cplx<double>>(), M, S, nvec, c->lrd.as<double>(), 1.0, st);
     }
-    launch_int_to_ext(Y, nvec, g.ld, c->npw_h, c->t_emap.as<int>(), c->t_econj.as<int>(), out, st);
+    launch_int_to_ext<double>(Y, nvec, g.ld, c->npw_h, c->t_emap.as<int>(), c->t_econj.as<int>(), out, st);
     WDF_CUDA_TRY(cudaStreamSynchronize(st));
     return WDF_OK;
   } catch (const ApiFailure &f) {
