@@ -121,11 +121,10 @@ template <typename S> void write_out(wdf_ctx *c, DBuf &stage, const cplx<S> *in,
 template <typename S = double>
 cplx<S> *read_in(wdf_ctx *c, DBuf &stage, DBuf &buf, const double *src, int n, int mem, int extra_rows = 0) {
   const double *d = stage_in(c, stage, src, 2 * (size_t)n * c->npw_h, mem);
-  const size_t bytes = sizeof(cplx<S>) * (size_t)(n + extra_rows) * c->geo.ld;
-  buf.ensure(bytes);
-  WDF_CUDA_TRY(cudaMemsetAsync(buf.p, 0, bytes, c->st));
-  launch_ext_to_int<S>(d, n, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr,
-                    buf.as<cplx<S>>(), c->geo.ld, c->st);
+  const size_t row = sizeof(cplx<S>) * (size_t)c->geo.ld;
+  buf.ensure(row * (size_t)(n + extra_rows));
+  if (extra_rows) WDF_CUDA_TRY(cudaMemsetAsync(buf.as<char>() + row * n, 0, row * extra_rows, c->st));
+  launch_ext_to_int<S>(d, n, c->npw_h, c->t_src.as<int>(), buf.as<cplx<S>>(), c->geo.ld, c->st);
   return buf.as<cplx<S>>();
 }
 
@@ -190,7 +189,12 @@ void setup_body(wdf_ctx *c, const wdf_system *sys) {
   upload(c, c->t_g2, L.g2);
   upload(c, c->t_vhalf, L.vhalf);
   upload(c, c->t_emap, L.emap);
-  upload(c, c->t_emap2, L.emap2);
+  std::vector<int> src(L.ld, -1);  // the inverse map: 2 i + (1 for the conjugate)
+  for (int i = 0; i < c->npw_h; ++i) {
+    src[L.emap[i]] = 2 * i + (L.econj[i] ? 1 : 0);
+    if (L.emap2[i] >= 0) src[L.emap2[i]] = 2 * i + (L.econj[i] ? 0 : 1);
+  }
+  upload(c, c->t_src, src);
   upload(c, c->t_econj, L.econj);
   // twiddles exp(2 pi i t / n) from long double sines and cosines
   std::vector<double> tw64;
@@ -283,8 +287,7 @@ void setup_body(wdf_ctx *c, const wdf_system *sys) {
   WDF_CUDA_TRY(cudaMemsetAsync(c->U64.p, 0, sizeof(cplx<double>) * (size_t)M * g.ld, c->st));
   if (c->nproj > 0) {
     const double *d = stage_in(c, c->ext_in, sys->beta, 2 * (size_t)c->nproj * c->npw_h, sys->mem);
-    launch_ext_to_int<double>(d, c->nproj, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr,
-                      c->U64.as<cplx<double>>(), g.ld, c->st);
+    launch_ext_to_int<double>(d, c->nproj, c->npw_h, c->t_src.as<int>(), c->U64.as<cplx<double>>(), g.ld, c->st);
   }
   c->lrd.ensure(sizeof(double) * M);
   {
@@ -304,8 +307,7 @@ void setup_body(wdf_ctx *c, const wdf_system *sys) {
   int status = WDF_OK;
   if (sys->psi) {
     const double *d = stage_in(c, c->ext_in, sys->psi, 2 * (size_t)c->nocc * c->npw_h, sys->mem);
-    launch_ext_to_int<double>(d, c->nocc, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr,
-                      c->U64.as<cplx<double>>() + (size_t)c->nproj * g.ld, g.ld, c->st);
+    launch_ext_to_int<double>(d, c->nocc, c->npw_h, c->t_src.as<int>(), c->U64.as<cplx<double>>() + (size_t)c->nproj * g.ld, g.ld, c->st);
     c->eps.assign(sys->eps, sys->eps + c->nocc);
     for (double e : c->eps)
       if (!std::isfinite(e)) throw ApiFailure(WDF_ENAN, "non-finite eigenvalue");
@@ -358,9 +360,7 @@ struct UserOp : DavOp {
     const int rc = fn(user, n, c->uop_in.as<double>(), c->uop_out.as<double>());
     if (rc != 0) throw ApiFailure(WDF_EINVAL, "the operator callback returned " + std::to_string(rc));
     ++calls;
-    const size_t bytes = sizeof(cplx<double>) * (size_t)n * c->geo.ld;
-    WDF_CUDA_TRY(cudaMemsetAsync(Y, 0, bytes, c->st));
-    launch_ext_to_int<double>(c->uop_out.as<double>(), n, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr, Y,
+    launch_ext_to_int<double>(c->uop_out.as<double>(), n, c->npw_h, c->t_src.as<int>(), Y,
                       c->geo.ld, c->st);
   }
 };
@@ -439,7 +439,7 @@ void wdf_destroy(wdf_ctx *c) {
   if (c->st) (void)cudaStreamSynchronize(c->st);
   else (void)cudaDeviceSynchronize();
   DBuf *bufs[] = {&c->t_col_off, &c->t_col_zlo, &c->t_e_col, &c->t_e_z,   &c->t_tile,  &c->t_xact,   &c->t_pos3,   &c->t_g2,
-                  &c->t_vhalf,   &c->t_emap,    &c->t_emap2, &c->t_econj, &c->t_tw64,  &c->t_tw32,   &c->vloc64,   &c->vloc32,   &c->vgroup32,
+                  &c->t_vhalf,   &c->t_emap,    &c->t_src, &c->t_econj, &c->t_tw64,  &c->t_tw32,   &c->vloc64,   &c->vloc32,   &c->vgroup32,
                   &c->U64,       &c->U32,       &c->lrd,     &c->psir64,  &c->psir32,  &c->kp64,     &c->kp32,     &c->tkin,
                   &c->eps_dev,   &c->rb,        &c->rx,      &c->rr,      &c->rAx,     &c->rwork,    &c->shift,    &c->vidx_dev,
                   &c->thr,       &c->gramw,     &c->xpert,   &c->dvgrid,  &c->accgrid, &c->cb2,      &c->outi,     &c->drhoi,

@@ -1151,48 +1151,40 @@ template <typename Tin, typename Tout> void launch_convert(const Geo &, Tout *y,
   WDF_CUDA_TRY(cudaGetLastError());
 }
 
-// External half-sphere vectors -> the internal layout, in FP64 or directly in double-float. A block takes
-// 256 coefficients of one row after the other (their map entries stay in registers). 512 rows of 23,168
-// take 189 us in double-float; with 64-bit divisions per coefficient and the split as a pass of its own
-// 142 + 172 us.
+// External half-sphere vectors -> the internal layout, in FP64 or directly in double-float: a gather by
+// src[e] = 2 i + (1 for the conjugate), -1 in the row padding. A block takes 256 elements of one row after
+// the other (their map entries stay in registers). Bound by HBM with the caller's rows re-read from L2:
+// 512 rows of 23,168 in double-float take 80 us; as a scatter, which writes 16-byte pieces and needs the
+// rows cleared first, 189 + 29 us.
 template <typename S>
-__global__ void __launch_bounds__(256) k_ext_to_int(const double *__restrict__ ext, int n, int npw_h, const int *__restrict__ emap,
-                             const int *__restrict__ emap2, const int *__restrict__ econj, const double *__restrict__ scale,
-                             cplx<S> *__restrict__ out, int ld) {
-  const int i = blockIdx.x * 256 + threadIdx.x;
-  if (i >= npw_h) return;
-  const int e = emap[i], e2 = emap2[i];
-  const bool conj = econj[i] != 0;
-  const double sc = scale ? scale[e] : 1.0;
+__global__ void __launch_bounds__(256) k_ext_to_int(const double *__restrict__ ext, int n, int npw_h, const int *__restrict__ src,
+                                                   cplx<S> *__restrict__ out, int ld) {
+  const int e = blockIdx.x * 256 + threadIdx.x;
+  if (e >= ld) return;
+  const int c = src[e], i = c >> 1;
 #pragma unroll 4
   for (int s = blockIdx.y; s < n; s += gridDim.y) {
-    const double *v = ext + 2 * ((size_t)s * npw_h + i);
-    double re = v[0], im = i == 0 ? 0.0 : v[1];  // G = 0 coefficient of a real function is real
-    if (conj) im = -im;
-    if (scale) {
-      re *= sc;
-      im *= sc;
+    double re = 0.0, im = 0.0;
+    if (c >= 0) {
+      const double *v = ext + 2 * ((size_t)s * npw_h + i);
+      re = v[0];
+      im = i == 0 ? 0.0 : v[1];  // G = 0 coefficient of a real function is real
+      if (c & 1) im = -im;
     }
-    const S x = cast<S>(re), y = cast<S>(im);
-    out[(size_t)s * ld + e] = mkc<S>(x, y);
-    if (e2 >= 0) out[(size_t)s * ld + e2] = mkc<S>(x, -y);
+    out[(size_t)s * ld + e] = mkc<S>(cast<S>(re), cast<S>(im));
   }
 }
-static dim3 ext_grid(int n, int npw_h) {
-  const int nb = (npw_h + 255) / 256;
+static dim3 ext_grid(int n, int len) {
+  const int nb = (len + 255) / 256;
   return dim3(nb, std::min(n, std::max(1, 16 * 152 / nb)));
 }
-template <typename S>
-void launch_ext_to_int(const double *ext, int n, int npw_h, const int *emap, const int *emap2, const int *econj,
-                       const double *scale_int, cplx<S> *out, int ld, cudaStream_t st) {
+template <typename S> void launch_ext_to_int(const double *ext, int n, int npw_h, const int *src, cplx<S> *out, int ld, cudaStream_t st) {
   if (n <= 0) return;
-  launch("ext_to_int", 0, k_ext_to_int<S>, ext_grid(n, npw_h), dim3(256), 0, st, ext, n, npw_h, emap, emap2, econj, scale_int, out, ld);
+  launch("ext_to_int", 0, k_ext_to_int<S>, ext_grid(n, ld), dim3(256), 0, st, ext, n, npw_h, src, out, ld);
   WDF_CUDA_TRY(cudaGetLastError());
 }
-template void launch_ext_to_int<double>(const double *, int, int, const int *, const int *, const int *, const double *, cplx<double> *, int,
-                                        cudaStream_t);
-template void launch_ext_to_int<df64>(const double *, int, int, const int *, const int *, const int *, const double *, cplx<df64> *, int,
-                                      cudaStream_t);
+template void launch_ext_to_int<double>(const double *, int, int, const int *, cplx<double> *, int, cudaStream_t);
+template void launch_ext_to_int<df64>(const double *, int, int, const int *, cplx<df64> *, int, cudaStream_t);
 
 template <typename S>
 __global__ void __launch_bounds__(256) k_int_to_ext(const cplx<S> *__restrict__ in, int n, int ld, int npw_h, const int *__restrict__ emap,

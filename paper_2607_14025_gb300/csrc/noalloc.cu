@@ -94,10 +94,9 @@ extern "C" int wdf_apply_hamiltonian_noalloc(wdf_ctx *c, int nvec, const double 
     double *S = reinterpret_cast<double *>(base + 2 * bx + bcb);
     double *gw = reinterpret_cast<double *>(base + 2 * bx + bcb + bs);
     double *zs = reinterpret_cast<double *>(base + 2 * bx + bcb + bs + bgw);
-    // the padding of X and the shifts must be zero; everything else is written before it is read
-    WDF_CUDA_TRY(cudaMemsetAsync(X, 0, bx, st));
+    // the shifts must be zero; everything else is written before it is read
     WDF_CUDA_TRY(cudaMemsetAsync(zs, 0, bz, st));
-    launch_ext_to_int<double>(in, nvec, c->npw_h, c->t_emap.as<int>(), c->t_emap2.as<int>(), c->t_econj.as<int>(), nullptr, X, g.ld, st);
+    launch_ext_to_int<double>(in, nvec, c->npw_h, c->t_src.as<int>(), X, g.ld, st);
     // H x = 1/2|G|^2 x + fft_n(V_loc ifft(x)) + sum_j beta_j D_j <beta_j, x>
     launch_zpass_g2r<double>(c->f64, X, nvec, cb, st);
     PlaneArgs<double> pa;
