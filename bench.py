@@ -97,12 +97,12 @@ ALU_PEAK_SOURCE = {"mixed_df": "FP32: 152 SMs x 128 lanes x 2 flop x 2070 MHz (d
 # DRAM bytes per (pair, z plane) unit of the FP32 V_loc plane kernel, per (grid, kernel variant
 # chosen at setup), from one ncu capture each on a small case of the same system
 # (dram__bytes_read.sum + dram__bytes_write.sum over the units of the captured launch; see
-# profiles/); traffic grows in proportion to the units launched. A variant without a capture of
-# its current code reports null.
+# profiles/); traffic grows in proportion to the units launched. The 64 value is that of the kernel's earlier form,
+# which copied the same slices. A variant without a capture reports null.
 PLANE_DRAM_BYTES_PER_UNIT = {
     (64, 1): (210.873088e6 + 167.385088e6) / 32768,  # k_plane_reg<64>: 32,768 units
-    (64, 5): (210.877440e6 + 149.595648e6) / 32768,  # k_plane_pipe<15>: 32,768 units
-    (96, 7): (311.997440e6 + 249.979648e6) / 24576,  # k_plane_pipe2<96, 22>: 24,576 units
+    (64, 5): (210.877440e6 + 149.595648e6) / 32768,  # k_plane_pipe<64, 15>: 32,768 units
+    (96, 5): (157.77e6 + 95.63e6) / 12288,  # k_plane_pipe<96, 22>: 12,288 units
 }
 
 
