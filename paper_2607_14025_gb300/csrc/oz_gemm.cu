@@ -552,13 +552,31 @@ int num_sms() {
   return nsm;
 }
 
-// K splits of the Gram: enough work items for the SMs, down to one chain (OZ_CHAIN stages) each, and at
-// most OZ_MAXCHAIN chains per split. With at least four chains a split the 192 x 3 products of the
-// 64^3 system ran in 16 CTAs of 66 stages (60 us); in 66 CTAs of 16 they take 26 us.
+// K splits of the Gram: at most OZ_MAXCHAIN chains each, at least one chain (OZ_CHAIN stages), and among
+// those the least estimated time of the persistent launch: its waves of work items, each the item's
+// stages and a quarter of a chain for its start and end, plus the pass that adds the partial sums (about
+// 1 us per split of 96 tiles, where a chain takes 11). The first split count whose items reach the number
+// of SMs, as chosen before, often starts a second wave that is nearly empty: 96 tiles (768 x 512 on 96^3)
+// in 2 splits are 192 items on 152 SMs, two waves of 46 chains, where 3 splits make two waves of 31
+// (1,018 -> 704 us); 21 tiles (366 x 201 on 75^3) in 8 splits are 168 items, two waves of 6 chains, in 7 one of 7
+// (148 -> 96 us). From four waves on the ragged one weighs little and there is nothing to choose. A split count
+// has to beat a smaller one by 5%, since each adds a partial sum.
 int gram_splits(int tiles, int nst) {
-  int nsplit = std::max(1, (nst + OZ_CHAIN * OZ_MAXCHAIN - 1) / (OZ_CHAIN * OZ_MAXCHAIN));
-  while (tiles * nsplit < num_sms() && nst / (nsplit + 1) >= OZ_CHAIN) ++nsplit;
-  return nsplit;
+  const int base = std::max(1, (nst + OZ_CHAIN * OZ_MAXCHAIN - 1) / (OZ_CHAIN * OZ_MAXCHAIN)), nsm = num_sms();
+  if (tiles >= 4 * nsm) return base;
+  auto cost = [&](int s) {
+    const int per = (nst + s - 1) / s, used = (nst + per - 1) / per;
+    const long waves = ((long)tiles * used + nsm - 1) / nsm;
+    return waves * (per + OZ_CHAIN / 4.0) + (double)used * tiles * OZ_CHAIN / (7.0 * nsm);
+  };
+  int best = base;
+  double tbest = cost(base);
+  for (int s = base + 1; s <= std::min(nst / OZ_CHAIN, base + std::max(16, nsm / tiles)); ++s)
+    if (cost(s) < 0.95 * tbest) {
+      best = s;
+      tbest = cost(s);
+    }
+  return best;
 }
 
 template <int T, int EPI>
