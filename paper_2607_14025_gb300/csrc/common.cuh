@@ -161,7 +161,7 @@ inline void launch(const char *cls, int bits, void (*k)(KArgs...), dim3 grid, di
 }
 
 // launch_units with programmatic stream serialisation: the grid may be set up while the kernel before it
-// in the stream finishes (that one calls pdl_begin first thing). A kernel launched this way calls pdl_wait
+// in the stream finishes (that one calls pdl_begin early). A kernel launched this way calls pdl_wait
 // in every thread before it touches memory that earlier work wrote and before it can exit, so that
 // its own completion implies the completion of everything before it. A chain of short kernels (the CG
 // iteration of a small system) hides the launch gaps and each kernel's prologue this way: 30^3 block 4.3
@@ -194,6 +194,11 @@ inline void launch_pdl(const char *cls, int bits, long long units, void (*k)(KAr
     t_prof->blocks += units;
   }
 }
+// Every CTA of a grid has called pdl_begin before a dependent CTA starts; one thread's call counts for its
+// CTA. A CTA calls it with everything in hand that it could have to wait for: tensor memory is allocated first, by
+// the same warp. Otherwise a dependent CTA could take the columns before its own pdl_wait and wait for
+// this grid, which waits for the columns (also across a kernel between the two, since that one
+// calls pdl_begin while it waits itself).
 __device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

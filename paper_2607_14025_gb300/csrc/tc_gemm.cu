@@ -104,8 +104,10 @@ __global__ void __launch_bounds__(kGramThreads, 1) k_gram_tc(const __grid_consta
     }
     tc::fence_mbar_init();
   }
-  pdl_begin();
-  if (warp == 0) tc::tmem_alloc(slot, 512);
+  if (warp == 0) {
+    tc::tmem_alloc(slot, 512);
+    pdl_begin();  // after the allocation: see pdl_begin
+  }
   tc::fence_before_sync();
   pdl_wait();
   __syncthreads();
@@ -295,8 +297,10 @@ __global__ void __launch_bounds__(256, 1) k_lincomb_tc(const __grid_constant__ C
     tc::mbar_init(done_bar, 1);
     tc::fence_mbar_init();
   }
-  pdl_begin();
-  if (warp == 0) tc::tmem_alloc(slot, 256);
+  if (warp == 0) {
+    tc::tmem_alloc(slot, 256);
+    pdl_begin();  // after the allocation: see pdl_begin
+  }
   tc::fence_before_sync();
   pdl_wait();
   __syncthreads();
