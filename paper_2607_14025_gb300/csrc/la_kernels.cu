@@ -951,7 +951,12 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
   const double rz = s.rz[i];
   pap = block_sum_all(pap, redp);
   if (!(pap > 0.0)) {  // breakdown: keep the current iterate (every block of the row sees the same sum)
-    if (c == 0 && threadIdx.x == 0) s.active[i] = 0;
+    // the last block to arrive stops the solve: cleared earlier, the flag could differ between the warps of a
+    // block that has just begun, and its sum of <p, A p> would lack those that left
+    if (threadIdx.x == 0 && (nchunk == 1 || atomicAdd(&s.arrived[i], 1) == nchunk - 1)) {
+      s.arrived[i] = 0;
+      s.active[i] = 0;
+    }
     return;
   }
   const T al = (T)(rz / pap);
