@@ -980,7 +980,10 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
         xe[q].y += al * pe[q].y;
         re[q].x -= al * ae[q].x;
         re[q].y -= al * ae[q].y;
-        if (eu + q >= e1) continue;  // an element of row padding (zero, and stays zero)
+        if (eu + q >= e1) {  // the element of row padding after an odd last one: p and A p hold anything there
+          xe[q] = re[q] = mkc<T>((T)0, (T)0);
+          continue;
+        }
         const T k = K ? ke[q] : (T)1;
         const cplx<T> zv = mkc<T>(k * re[q].x, k * re[q].y);  // z = K r, recomputed where it is needed
         const A w = eu + q < g.len0 ? (A)1 : (A)2;

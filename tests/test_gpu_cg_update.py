@@ -113,3 +113,15 @@ def test_breakdown_stops_the_solve_and_keeps_its_iterate(lib, nint, n):
     go = [i for i in range(n) if i not in (1, 2)]
     assert np.all(a["active"][go] == 1) and np.all(a["iters"][go] == 1) and not np.array_equal(a["x"][0], before["x"][0])
     assert np.all(a["arrived"] == 0) and list(a["nactive"]) == [0, n - 2]
+
+
+@pytest.mark.parametrize("nint,n", [(447, 5), (2049, 3), (8455, 5), (8455, 700)])
+def test_row_padding_stays_zero(lib, nint, n):
+    """The padding of p and A p is never written by the library, so that of x and r must not depend on it."""
+    b = Batch(nint, n)
+    b.p[:, nint:] = float("nan")
+    b.Ap[:, nint:] = float("nan")
+    a = b.step(lib)
+    for k in ("x", "r"):
+        assert np.all(a[k][:, nint:] == 0.0) and np.isfinite(a[k]).all()
+    assert np.isfinite(a["rr"]).all() and np.isfinite(a["rz"]).all()
