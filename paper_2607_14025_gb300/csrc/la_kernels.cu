@@ -919,7 +919,7 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
   typedef typename UpdVec<T>::K KV;
   constexpr int E = UpdVec<T>::E, UB = 2, STEP = 256 * E * UB;
   const int i = blockIdx.x, c = blockIdx.y;
-  __shared__ double redp[8], red3[3][8];
+  __shared__ double redp[8], red3[3][8], fold[3][256];
   pdl_begin();
   pdl_wait();
   if (i == 0 && c == 0 && threadIdx.x == 0) s.nactive[which ^ 1] = 0;  // the next launch's count
@@ -960,7 +960,11 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
     return;
   }
   const T al = (T)(rz / pap);
+  // a thread's sums over DCHUNK elements of the row are FP32 in an FP32 solve and are added up in FP64 (in
+  // shared memory: the registers are all in use), so a block of four times as many loses nothing
   A vrz = 0, vrr = 0, vr3 = 0;
+  const int t = threadIdx.x;
+  fold[0][t] = fold[1][t] = fold[2][t] = 0.0;
   for (; e < e1; e += STEP, load(e)) {
 #pragma unroll
     for (int u = 0; u < UB; ++u) {
@@ -995,8 +999,14 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
       *reinterpret_cast<V *>(x + ox + eu) = upd_vec(xe);
       *reinterpret_cast<V *>(r + o + eu) = upd_vec(re);
     }
+    if ((e & (DCHUNK - 1)) >= DCHUNK - STEP) {  // e0 is a multiple of DCHUNK
+      fold[0][t] += (double)vrz;
+      fold[1][t] += (double)vrr;
+      if (fb) fold[2][t] += (double)vr3;
+      vrz = vrr = vr3 = 0;
+    }
   }
-  double sum[3] = {(double)vrz, (double)vrr, (double)vr3};
+  double sum[3] = {fold[0][t] + (double)vrz, fold[1][t] + (double)vrr, fold[2][t] + (double)vr3};
   block_sum3(sum, fb, red3);
   if (threadIdx.x != 0) return;
   if (nchunk > 1) {  // the last block of the row to arrive adds the chunks in order
@@ -1041,7 +1051,7 @@ template <typename T>
 void launch_cg_update(const Geo &g, cplx<T> *x, cplx<T> *r, const cplx<T> *p, const cplx<T> *Ap, const T *kprec, const CgState &s, int n,
                       const double *dots, int ndot, int maxiter, int which, cudaStream_t st) {
   if (n <= 0) return;
-  // DCHUNK elements a block; four times as many once that still leaves four blocks for each of the
+  // DCHUNK (a power of two) elements a block; four times as many once that still leaves four blocks for each of the
   // 152 SMs twice over, so that a block's start and sums weigh less
   const int chunk = (long)n * ((g.nint + 4 * DCHUNK - 1) / (4 * DCHUNK)) >= 8 * 152 ? 4 * DCHUNK : DCHUNK;
   const int nchunk = (g.nint + chunk - 1) / chunk;

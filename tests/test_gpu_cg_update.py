@@ -125,3 +125,19 @@ def test_row_padding_stays_zero(lib, nint, n):
     for k in ("x", "r"):
         assert np.all(a[k][:, nint:] == 0.0) and np.isfinite(a[k]).all()
     assert np.isfinite(a["rr"]).all() and np.isfinite(a["rz"]).all()
+
+
+@pytest.mark.parametrize("nint", [2048, 8455, 23171])
+def test_sums_do_not_depend_on_the_size_of_the_batch(lib, nint):
+    """<r, K r> and <r, r> of a row alone and in a batch whose blocks take four times as many elements.
+
+    Both add the same FP32 sums of at most 8 elements, all positive, in FP64 and in another order: at most
+    256 ceil(nint / 2048) additions of relative error 2^-53 each.
+    """
+    n = 8 * 152 // ((nint + 8191) // 8192) + 1
+    one, many = Batch(nint, 1).step(lib), Batch(nint, n).step(lib)
+    bar = 256 * ((nint + 2047) // 2048) * 2.0 ** -53
+    for k in ("rz", "rr"):
+        assert np.all(many[k] == many[k][0])
+        assert abs(many[k][0] - one[k][0]) <= bar * one[k][0]
+    assert np.array_equal(many["x"][0], one["x"][0]) and np.array_equal(many["r"][0], one["r"][0])
