@@ -113,7 +113,7 @@ template <typename S> void write_out(wdf_ctx *c, DBuf &stage, const cplx<S> *in,
     stage.ensure(nd * sizeof(double));
     target = stage.as<double>();
   }
-  launch_int_to_ext<S>(in, n, c->geo.ld, c->npw_h, c->t_emap.as<int>(), c->t_econj.as<int>(), target, c->st);
+  launch_int_to_ext<S>(in, n, c->geo.ld, c->npw_h, c->t_emap.as<int>(), target, c->st);
   if (mem == WDF_MEM_HOST) WDF_CUDA_TRY(cudaMemcpyAsync(dst, target, nd * sizeof(double), cudaMemcpyDeviceToHost, c->st));
 }
 
@@ -188,14 +188,14 @@ void setup_body(wdf_ctx *c, const wdf_system *sys) {
   upload(c, c->t_pos3, L.pos3);
   upload(c, c->t_g2, L.g2);
   upload(c, c->t_vhalf, L.vhalf);
-  upload(c, c->t_emap, L.emap);
-  std::vector<int> src(L.ld, -1);  // the inverse map: 2 i + (1 for the conjugate)
+  std::vector<int> dst(c->npw_h), src(L.ld, -1);  // 2 e + (1 for the conjugate); the inverse map: 2 i + (1 likewise)
   for (int i = 0; i < c->npw_h; ++i) {
+    dst[i] = 2 * L.emap[i] + (L.econj[i] ? 1 : 0);
     src[L.emap[i]] = 2 * i + (L.econj[i] ? 1 : 0);
     if (L.emap2[i] >= 0) src[L.emap2[i]] = 2 * i + (L.econj[i] ? 0 : 1);
   }
+  upload(c, c->t_emap, dst);
   upload(c, c->t_src, src);
-  upload(c, c->t_econj, L.econj);
   // twiddles exp(2 pi i t / n) from long double sines and cosines
   std::vector<double> tw64;
   std::vector<float> tw32;
@@ -354,7 +354,7 @@ struct UserOp : DavOp {
     const size_t nd = 2 * (size_t)n * c->npw_h;
     c->uop_in.ensure(nd * sizeof(double));
     c->uop_out.ensure(nd * sizeof(double));
-    launch_int_to_ext<double>(X, n, c->geo.ld, c->npw_h, c->t_emap.as<int>(), c->t_econj.as<int>(), c->uop_in.as<double>(), c->st);
+    launch_int_to_ext<double>(X, n, c->geo.ld, c->npw_h, c->t_emap.as<int>(), c->uop_in.as<double>(), c->st);
     WDF_CUDA_TRY(cudaMemsetAsync(c->uop_out.p, 0, nd * sizeof(double), c->st));
     WDF_CUDA_TRY(cudaStreamSynchronize(c->st));  // the callback may work on any stream
     const int rc = fn(user, n, c->uop_in.as<double>(), c->uop_out.as<double>());
@@ -439,7 +439,7 @@ void wdf_destroy(wdf_ctx *c) {
   if (c->st) (void)cudaStreamSynchronize(c->st);
   else (void)cudaDeviceSynchronize();
   DBuf *bufs[] = {&c->t_col_off, &c->t_col_zlo, &c->t_e_col, &c->t_e_z,   &c->t_tile,  &c->t_xact,   &c->t_pos3,   &c->t_g2,
-                  &c->t_vhalf,   &c->t_emap,    &c->t_src, &c->t_econj, &c->t_tw64,  &c->t_tw32,   &c->vloc64,   &c->vloc32,   &c->vgroup32,
+                  &c->t_vhalf,   &c->t_emap,    &c->t_src, &c->t_tw64,  &c->t_tw32,   &c->vloc64,   &c->vloc32,   &c->vgroup32,
                   &c->U64,       &c->U32,       &c->lrd,     &c->psir64,  &c->psir32,  &c->kp64,     &c->kp32,     &c->tkin,
                   &c->eps_dev,   &c->rb,        &c->rx,      &c->rr,      &c->rAx,     &c->rwork,    &c->shift,    &c->vidx_dev,
                   &c->thr,       &c->gramw,     &c->xpert,   &c->dvgrid,  &c->accgrid, &c->cb2,      &c->outi,     &c->drhoi,

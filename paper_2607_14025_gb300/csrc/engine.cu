@@ -1417,6 +1417,14 @@ void finish_setup(wdf_ctx *c) {
     c->f32.vgroup = c->vgroup32.as<float>();
   }
   autotune_vloc<float>(c, c->f32, c->vloc32.as<float>());
+  // one FP32 copy is kept, in the order that the chosen kernel reads: a context holds no more than with the
+  // natural order alone, and setup's peak stays the column buffer of the FP64-class timing below
+  if (c->f32.vloc_variant == 5 || c->f32.vloc_variant == 8) {
+    c->vloc32.release();
+  } else {
+    c->f32.vgroup = nullptr;
+    c->vgroup32.release();
+  }
   if (c->opt.precision == WDF_MIXED_DF) autotune_vloc<df64>(c, c->fdf, c->vlocdf.as<df64>());
   else autotune_vloc<double>(c, c->f64, c->vloc64.as<double>());
   WDF_CUDA_TRY(cudaStreamSynchronize(st));

@@ -67,10 +67,10 @@ struct wdf_ctx {
 
   // layout tables
   wdf::DBuf t_col_off, t_col_zlo, t_e_col, t_e_z, t_tile, t_xact, t_pos3, t_g2, t_vhalf;
-  wdf::DBuf t_emap, t_src, t_econj, t_tw64, t_tw32, t_twdf, t_xactn, t_jidx, t_jnat;
+  wdf::DBuf t_emap, t_src, t_tw64, t_tw32, t_twdf, t_xactn, t_jidx, t_jnat;
 
   // operator data
-  wdf::DBuf vloc64, vloc32, vgroup32;  // V_loc on the grid
+  wdf::DBuf vloc64, vloc32, vgroup32;  // V_loc on the grid (FP32: in one of the two orders, see finish_setup)
   wdf::DBuf U64, U32;        // [nproj + nocc][ld]: projectors then occupied orbitals (internal layout)
   wdf::DBuf lrd;             // [nproj + nocc]: D_j then alpha
   wdf::DBuf psir64, psir32;  // [nocc][ngrid] psi_v(r) (unnormalised inverse transform)

@@ -206,11 +206,11 @@ template <typename T> void launch_scale_rows(const Geo &g, cplx<T> *y, const dou
 template <typename Tin, typename Tout>
 void launch_convert(const Geo &g, Tout *y, const Tin *x, size_t count, cudaStream_t st);
 // external half-sphere vectors <-> internal layout (S: FP64 or double-float)
-// out: whole rows, the padding written as zeros; src (ld entries): 2 i + (1: conjugate), or -1
+// out: whole rows, the padding written as zeros; src (ld entries): 2 i + (1: conjugate), or -1; emap (npw_h
+// entries): 2 e + (1: conjugate)
 template <typename S> void launch_ext_to_int(const double *ext, int n, int npw_h, const int *src, cplx<S> *out, int ld, cudaStream_t st);
 template <typename S>
-void launch_int_to_ext(const cplx<S> *in, int n, int ld, int npw_h, const int *emap, const int *econj,
-                       double *ext, cudaStream_t st);
+void launch_int_to_ext(const cplx<S> *in, int n, int ld, int npw_h, const int *emap, double *ext, cudaStream_t st);
 // residual subtraction for Davidson: R_a = AX_a - theta_a X_a
 void launch_ritz_residual(const Geo &g, cplx<double> *R, const cplx<double> *AX, const cplx<double> *X,
                           const double *theta, int n, cudaStream_t st);

@@ -1206,11 +1206,11 @@ template void launch_ext_to_int<df64>(const double *, int, int, const int *, cpl
 
 template <typename S>
 __global__ void __launch_bounds__(256) k_int_to_ext(const cplx<S> *__restrict__ in, int n, int ld, int npw_h, const int *__restrict__ emap,
-                             const int *__restrict__ econj, double *__restrict__ ext) {
+                             double *__restrict__ ext) {
   const int i = blockIdx.x * 256 + threadIdx.x;
   if (i >= npw_h) return;
-  const int e = emap[i];
-  const bool conj = econj[i] != 0;
+  const int e = emap[i] >> 1;
+  const bool conj = emap[i] & 1;
 #pragma unroll 4
   for (int s = blockIdx.y; s < n; s += gridDim.y) {
     const cplx<S> v = in[(size_t)s * ld + e];
@@ -1221,14 +1221,14 @@ __global__ void __launch_bounds__(256) k_int_to_ext(const cplx<S> *__restrict__ 
   }
 }
 template <typename S>
-void launch_int_to_ext(const cplx<S> *in, int n, int ld, int npw_h, const int *emap, const int *econj, double *ext,
+void launch_int_to_ext(const cplx<S> *in, int n, int ld, int npw_h, const int *emap, double *ext,
                        cudaStream_t st) {
   if (n <= 0) return;
-  launch("int_to_ext", 0, k_int_to_ext<S>, ext_grid(n, npw_h), dim3(256), 0, st, in, n, ld, npw_h, emap, econj, ext);
+  launch("int_to_ext", 0, k_int_to_ext<S>, ext_grid(n, npw_h), dim3(256), 0, st, in, n, ld, npw_h, emap, ext);
   WDF_CUDA_TRY(cudaGetLastError());
 }
-template void launch_int_to_ext<double>(const cplx<double> *, int, int, int, const int *, const int *, double *, cudaStream_t);
-template void launch_int_to_ext<df64>(const cplx<df64> *, int, int, int, const int *, const int *, double *, cudaStream_t);
+template void launch_int_to_ext<double>(const cplx<double> *, int, int, int, const int *, double *, cudaStream_t);
+template void launch_int_to_ext<df64>(const cplx<df64> *, int, int, int, const int *, double *, cudaStream_t);
 
 __global__ void k_ritz_residual(Geo g, cplx<double> *__restrict__ R, const cplx<double> *__restrict__ AX,
                                 const cplx<double> *__restrict__ X, const double *__restrict__ theta, int n) {

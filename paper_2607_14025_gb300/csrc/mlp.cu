@@ -343,7 +343,7 @@ __global__ void k_mlp_samples(Geo g, const int *__restrict__ emap, int npw_h, in
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)nocc * npw_h) return;
   const int v = (int)(t / npw_h), i = (int)(t % npw_h);
-  const int e = emap[i];
+  const int e = emap[i] >> 1;
   const size_t o = (size_t)v * g.ld + e, plane = (size_t)nocc * g.ld;
   float f[4];
   sample_features(g, e, tkin[v], eps[v], psi[o], (double)npw_h, f);

@@ -113,7 +113,7 @@ extern "C" int wdf_apply_hamiltonian_noalloc(wdf_ctx *c, int nvec, const double 
       launch_gram<double>(g, c->U64.as<cplx<double>>(), M, X, nvec, S, nvec, gw, bgw / sizeof(double), st);
       launch_lincomb<double>(g, Y, nvec, c->U64.as<cplx<double>>(), M, S, nvec, c->lrd.as<double>(), 1.0, st);
     }
-    launch_int_to_ext<double>(Y, nvec, g.ld, c->npw_h, c->t_emap.as<int>(), c->t_econj.as<int>(), out, st);
+    launch_int_to_ext<double>(Y, nvec, g.ld, c->npw_h, c->t_emap.as<int>(), out, st);
     WDF_CUDA_TRY(cudaStreamSynchronize(st));
     return WDF_OK;
   } catch (const ApiFailure &f) {
