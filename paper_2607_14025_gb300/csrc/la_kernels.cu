@@ -960,11 +960,11 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
     return;
   }
   const T al = (T)(rz / pap);
-  // a thread's sums over DCHUNK elements of the row are FP32 in an FP32 solve and are added up in FP64 (in
-  // shared memory: the registers are all in use), so a block of four times as many loses nothing
+  // a thread's sums over DCHUNK elements of the row are FP32 in an FP32 solve; a block that takes more adds them
+  // up in FP64 (in shared memory: the registers are all in use)
   A vrz = 0, vrr = 0, vr3 = 0;
   const int t = threadIdx.x;
-  fold[0][t] = fold[1][t] = fold[2][t] = 0.0;
+  const bool more = e + DCHUNK < e1;
   for (; e < e1; e += STEP, load(e)) {
 #pragma unroll
     for (int u = 0; u < UB; ++u) {
@@ -999,14 +999,20 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
       *reinterpret_cast<V *>(x + ox + eu) = upd_vec(xe);
       *reinterpret_cast<V *>(r + o + eu) = upd_vec(re);
     }
-    if ((e & (DCHUNK - 1)) >= DCHUNK - STEP) {  // e0 is a multiple of DCHUNK
-      fold[0][t] += (double)vrz;
-      fold[1][t] += (double)vrr;
-      if (fb) fold[2][t] += (double)vr3;
+    if (more && (e & (DCHUNK - 1)) >= DCHUNK - STEP && e + STEP < e1) {  // e0 is a multiple of DCHUNK
+      const bool first = e - e0 < DCHUNK;
+      fold[0][t] = first ? cast<double>(vrz) : fold[0][t] + cast<double>(vrz);
+      fold[1][t] = first ? cast<double>(vrr) : fold[1][t] + cast<double>(vrr);
+      if (fb) fold[2][t] = first ? cast<double>(vr3) : fold[2][t] + cast<double>(vr3);
       vrz = vrr = vr3 = 0;
     }
   }
-  double sum[3] = {fold[0][t] + (double)vrz, fold[1][t] + (double)vrr, fold[2][t] + (double)vr3};
+  double sum[3] = {cast<double>(vrz), cast<double>(vrr), fb ? cast<double>(vr3) : 0.0};
+  if (more) {
+    sum[0] += fold[0][t];
+    sum[1] += fold[1][t];
+    if (fb) sum[2] += fold[2][t];
+  }
   block_sum3(sum, fb, red3);
   if (threadIdx.x != 0) return;
   if (nchunk > 1) {  // the last block of the row to arrive adds the chunks in order
