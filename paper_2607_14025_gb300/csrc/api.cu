@@ -451,7 +451,7 @@ void wdf_destroy(wdf_ctx *c) {
                   &c->ml64,      &c->ml32,      &c->mlw64,   &c->krow,     &c->rr_ref,  &c->it_ref,  &c->nfb,
                   &c->mlsums,    &c->mlwraw,    &c->tcU,     &c->tcUt,     &c->tcC,     &c->tcerr,
                   &c->wp_phi,    &c->wp_x,      &c->wp_y,    &c->wp_vx,    &c->wp_S,    &c->wp_coef,
-                  &c->uop_in,    &c->uop_out,   &c->orbfields, &c->ones64,  &c->onesdf,  &c->pnorm,
+                  &c->uop_in,    &c->uop_out,   &c->orbfields, &c->pnorm,
                   &c->ozU,       &c->ozUe,      &c->ozUt,    &c->ozUte,    &c->ozPt,    &c->ozPte,   &c->ozX,
                   &c->ozXe,      &c->ozC,       &c->ozCe};
   for (DBuf *b : bufs) b->release();

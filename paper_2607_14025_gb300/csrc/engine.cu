@@ -169,16 +169,12 @@ template <> struct Stage<double> {
   static DBuf &dv(wdf_ctx *c) { return c->dvgrid; }
   static DBuf &acc(wdf_ctx *c) { return c->accgrid; }
   static DBuf &cb2(wdf_ctx *c) { return c->cb2; }
-  static DBuf &fields(wdf_ctx *c) { return c->orbfields; }
-  static DBuf &ones(wdf_ctx *c) { return c->ones64; }
 };
 template <> struct Stage<df64> {
   static const df64 *psir(wdf_ctx *c) { return c->psirdf.as<df64>(); }
   static DBuf &dv(wdf_ctx *c) { return c->dvgriddf; }
   static DBuf &acc(wdf_ctx *c) { return c->accgriddf; }
   static DBuf &cb2(wdf_ctx *c) { return c->cb2df; }
-  static DBuf &fields(wdf_ctx *c) { return c->orbfields; }
-  static DBuf &ones(wdf_ctx *c) { return c->onesdf; }
 };
 
 // FP64 complex vectors <-> double-float complex vectors (n rows of ld)
@@ -822,12 +818,41 @@ void sternheimer_solve(wdf_ctx *c, const cplx<double> *b, cplx<double> *x, const
 // ---------------------------------------------------------------------------------------------
 // chi0bar by DFPT (paper Sec. 2.1). phi: npert internal FP64 vectors (G = 0 ignored).
 
+// Orbitals whose real-space fields (one perturbation pair's, `real` bytes a real number) are held at once in the
+// density response, and the buffer: psi = 1 on the grid first, the fields `head` bytes on. The
+// refinement's A x (two rows per pair and orbital) is idle by then and holds one orbital's fields in 15 for each
+// pair (a row is a 31st of the grid on the model spheres): all of them from 16 pairs on. Blocks of
+// few solves have a buffer of their own of at most 64 MB. Memory that cannot be had is no error: 0 means the kernels that sum in place, which need
+// none (64 orbitals on 64^3, 2,048 solves: 4.5 ms against 3.0). Under a limit on the library's memory
+// the buffer is given back at once. (With all fields in a buffer of their own, 268 MB for those 64 orbitals,
+// calls were refused under limits that had been enough for the sum in place.)
+static int orbital_group(wdf_ctx *c, size_t real, DBuf **space, size_t &head) {
+  constexpr int kFew = 8;
+  constexpr size_t kOwnBytes = (size_t)64 << 20;
+  const size_t field = 2 * real * c->ngrid;
+  head = (real * c->ngrid + 255) / 256 * 256;
+  auto room = [&](size_t bytes) { return bytes > head ? (int)std::min<size_t>(c->nocc, (bytes - head) / field) : 0; };
+  int group = room(c->rAx.cap);
+  *space = &c->rAx;
+  if (group < std::min(c->nocc, kFew)) {
+    const int own = std::min(c->nocc, std::max(1, room(kOwnBytes)));
+    if (own > group && c->orbfields.try_ensure(head + field * own)) {
+      group = own;
+      *space = &c->orbfields;
+    }
+  }
+  if (group == 0) return 0;
+  const int ngroup = (c->nocc + group - 1) / group;
+  return (c->nocc + ngroup - 1) / ngroup;  // even groups
+}
+
 // Stages S2, S3, S7, S8 in R (FP64 or double-float); xp: np2 rows of v^1/2 phi (FP64). Results
 // (np2 rows, FP64) go to ou = v^1/2 drho and dr = drho.
 template <typename R>
 static void chi0_stages(wdf_ctx *c, const cplx<double> *xp64, int npert, const std::vector<char> &zero, cplx<double> *ou,
                         cplx<double> *dr, SolveStats &ss) {
   constexpr bool DF = std::is_same<R, df64>::value;
+  if (g_dev_cap.load() > 0) c->orbfields.release();
   const Geo &g = c->geo;
   cudaStream_t st = c->st;
   const FftCtx<R> &f = Prec<R>::f(c);
@@ -945,26 +970,29 @@ static void chi0_stages(wdf_ctx *c, const cplx<double> *xp64, int npert, const s
     cb2.ensure(sizeof(cplx<R>) * (size_t)(pp1 - pp0) * cbpair);
     accb.ensure(sizeof(cplx<R>) * (size_t)(pp1 - pp0) * ngrid);
     launch_zpass_g2r<R>(f, xR, ns, cb, st);
-    if (plane_accum_by_g2r<R>(f)) {
-      // per perturbation pair: every orbital's pair to real space (compile-time plane kernel), then
-      // the sum over orbitals on the grid; then the summed grids back to their column buffers
-      // (the product kernel with psi = 1)
-      DBuf &fields = Stage<R>::fields(c), &ones = Stage<R>::ones(c);
-      fields.ensure(sizeof(cplx<R>) * (size_t)nocc * ngrid);
-      if (ones.cap < sizeof(R) * ngrid) {
-        ones.ensure(sizeof(R) * ngrid);
-        launch_fill<R>(ones.as<R>(), ngrid, 1.0, st);
-      }
-      for (int pp = pp0; pp < pp1; ++pp) {
-        PlaneArgs<R> pg;
-        pg.cb = cb + (size_t)(pp - pp0) * nocc * cbpair;
-        pg.grid = fields.as<cplx<R>>();
-        launch_plane<R>(f, OP_G2R, nocc, pg, st);
-        launch_orbital_sum<R>(fields.as<cplx<R>>(), Stage<R>::psir(c), nocc, ngrid, accb.as<cplx<R>>() + (size_t)(pp - pp0) * ngrid, st);
-      }
+    size_t head = 0;
+    DBuf *space = nullptr;
+    const int group = plane_accum_by_g2r<R>(f) ? orbital_group(c, sizeof(R), &space, head) : 0;
+    if (group > 0) {
+      // per perturbation pair, a group of orbitals at a time: their pairs to real space (compile-time
+      // plane kernel), then added to the sum over orbitals on the grid, in order; then the summed
+      // grids back to their column buffers (the product kernel with psi = 1)
+      R *ones = space->as<R>();
+      cplx<R> *fields = reinterpret_cast<cplx<R> *>(space->as<char>() + head);
+      launch_fill<R>(ones, ngrid, 1.0, st);
+      for (int pp = pp0; pp < pp1; ++pp)
+        for (int v0 = 0; v0 < nocc; v0 += group) {
+          const int nv = std::min(group, nocc - v0);
+          PlaneArgs<R> pg;
+          pg.cb = cb + ((size_t)(pp - pp0) * nocc + v0) * cbpair;
+          pg.grid = fields;
+          launch_plane<R>(f, OP_G2R, nv, pg, st);
+          launch_orbital_sum<R>(fields, Stage<R>::psir(c) + (size_t)v0 * ngrid, nv, ngrid, accb.as<cplx<R>>() + (size_t)(pp - pp0) * ngrid,
+                                v0 == 0, st);
+        }
       PlaneArgs<R> pb;
       pb.cb = cb2.as<cplx<R>>();
-      pb.field = ones.as<R>();
+      pb.field = ones;
       pb.grid = accb.as<cplx<R>>();
       pb.nocc = 1;
       launch_plane<R>(f, OP_PROD_R2G, pp1 - pp0, pb, st);
@@ -984,6 +1012,7 @@ static void chi0_stages(wdf_ctx *c, const cplx<double> *xp64, int npert, const s
     ea.scale = R(4.0 / (c->omega * (double)ngrid));
     launch_zpass_r2g<R>(f, EPI_DRHO, cb2.as<cplx<R>>(), 2 * (pp1 - pp0), ea, st);
   }
+  if (g_dev_cap.load() > 0) c->orbfields.release();
   if constexpr (DF) {
     from_df(c, dr, drR, np2);
     from_df(c, ou, ouR, np2);

@@ -14,6 +14,7 @@ struct DBuf {
   size_t cap = 0;
   template <class T> T *as() const { return static_cast<T *>(p); }
   void ensure(size_t bytes);
+  bool try_ensure(size_t bytes);  // false where ensure() would throw WDF_ENOMEM
   void release();
 };
 // device bytes held by all DBufs of the process, cudaMalloc calls made for them, and the cap
@@ -111,7 +112,7 @@ struct wdf_ctx {
   wdf::DBuf wp_phi, wp_x, wp_y, wp_vx, wp_S, wp_coef;  // wdf_apply_wp
   wdf::DBuf uop_in, uop_out;                           // wdf_davidson: the caller's operator's in / out
   wdf::DBuf pnorm;                      // squared norms of a block's perturbations
-  wdf::DBuf orbfields, ones64, onesdf;  // orbital sum by G2R: one pair's real-space fields per orbital; psi = 1 grids
+  wdf::DBuf orbfields;                  // orbital sum by G2R in small blocks: one pair's real-space fields of a group of orbitals
   bool collect = false;
   wdf::DBuf rb, rx, rr, rAx, rwork;        // refinement: b, x, r, A x (FP64), FP32 staging
   wdf::DBuf shift, vidx_dev, thr;          // per-solve shift, orbital index, thresholds

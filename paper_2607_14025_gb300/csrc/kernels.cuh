@@ -55,9 +55,9 @@ template <typename T> bool plane_variant_available(const FftCtx<T> &f, int v);
 constexpr int kPlaneVariants = 8;  // variants are numbered 1 .. kPlaneVariants
 // whether the orbital sum of the density response runs as G2R transforms + k_orbital_sum
 template <typename T> bool plane_accum_by_g2r(const FftCtx<T> &f);
-// acc[i] = sum_v psir[v][i] fields[v][i] over the ngrid points, orbitals in order
+// acc[i] (+)= sum_v psir[v][i] fields[v][i] over the ngrid points, orbitals in order; first: acc starts here
 template <typename R>
-void launch_orbital_sum(const cplx<R> *fields, const R *psir, int nocc, size_t ngrid, cplx<R> *acc, cudaStream_t st);
+void launch_orbital_sum(const cplx<R> *fields, const R *psir, int nocc, size_t ngrid, cplx<R> *acc, bool first, cudaStream_t st);
 // x[i] = value
 template <typename R> void launch_fill(R *x, size_t count, double value, cudaStream_t st);
 // persistent FP32 V_loc plane kernel (plane_pipe.cu); false when the geometry has no instance

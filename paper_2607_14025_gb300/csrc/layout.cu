@@ -47,6 +47,15 @@ void DBuf::ensure(size_t bytes) {
   cap = bytes;
 }
 
+bool DBuf::try_ensure(size_t bytes) {
+  try {
+    ensure(bytes);
+    return true;
+  } catch (const ApiFailure &) {
+    return false;
+  }
+}
+
 void DBuf::release() {
   if (p) {
     (void)cudaFree(p);

@@ -400,9 +400,9 @@ template <typename T> void set_plane_fast_limits(const Geo &g) {
 template <typename T> bool launch_plane_fast(const FftCtx<T> &f, int op, int nblk, const PlaneArgs<T> &pa, cudaStream_t st) {
   const int v = op == OP_VLOC ? f.vloc_variant : 0;  // chosen at setup by timing (0: this order)
   if constexpr (std::is_same<T, df64>::value) {
-    // the one-task-per-thread 64 x 64 kernel: the orbital sum, V_loc (variant 6) and the product for bands
-    // that the line-resident kernel does not take
-    const bool use = !lines_chosen(f) && (op == OP_VLOC ? v == 6 : op == OP_ACCUM || op == OP_PROD_R2G);
+    // the one-task-per-thread 64 x 64 kernel: the orbital sum in place, and V_loc (variant 6) and the product
+    // for bands that the line-resident kernel does not take
+    const bool use = op == OP_ACCUM || (!lines_chosen(f) && (op == OP_VLOC ? v == 6 : op == OP_PROD_R2G));
     if (use && launch_plane_df(f, op, nblk, pa, st)) return true;
   }
   // the orbital sum of the density response keeps two register blocks across its loop and
@@ -455,7 +455,7 @@ template <typename T> bool plane_variant_available(const FftCtx<T> &f, int v) {
 }
 // the orbital sum of the density response as compile-time G2R transforms of each orbital's pair
 // followed by a separate sum over orbitals (k_orbital_sum): FP64-class arithmetic on grids with a
-// compile-time Stockham or line-resident kernel; 64 x 64 double-float planes without the latter sum in
+// compile-time Stockham or line-resident kernel, memory permitting (orbital_group); 64 x 64 double-float planes without the latter sum in
 // place in their own kernel (2,048 solves: 4.5 ms in place, 3.0 ms as line-resident transforms and a sum)
 template <typename T> bool plane_accum_by_g2r(const FftCtx<T> &f) {
   if constexpr (std::is_same<T, float>::value) {
