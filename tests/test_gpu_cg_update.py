@@ -74,7 +74,7 @@ class Batch:
         def rows():
             a = np.zeros((1, ld, 2), np.float32)
             a[:, :nint] = rng.standard_normal((1, nint, 2))
-            return torch.from_numpy(np.ascontiguousarray(np.broadcast_to(a, (n, ld, 2)))).cuda()
+            return torch.from_numpy(np.repeat(a, n, axis=0)).cuda()
 
         def dev(a):
             return torch.from_numpy(np.ascontiguousarray(a)).cuda()
