@@ -379,7 +379,9 @@ int wdf_profile_units(wdf_ctx *ctx, int64_t *blocks);
 /* The V_loc plane kernel chosen at setup by timing for the given arithmetic (bits = 32 FP32,
  * 64 FP64, 48 double-float): 1 register lines, 2 Stockham, 3 generic, 4 two-thread register
  * lines, 5 persistent with bulk copies, 6 double-float 64 x 64, 8 line-resident; 0 when that
- * arithmetic has no V_loc plane kernel in this context (WDF_EINVAL for other bits). Instrumentation: lets a caller match kernel counters taken
+ * arithmetic has no V_loc plane kernel in this context (WDF_EINVAL for other bits). 6 is two kernels:
+ * the line-resident one (that of 8) while the occupied columns lie in |n1|, |n2| <= 16, and for wider
+ * bands one with a transform task per thread. Instrumentation: lets a caller match kernel counters taken
  * on one variant to the kernel that runs. */
 int wdf_plane_variant(const wdf_ctx *ctx, int bits, int *variant);
 

@@ -436,7 +436,11 @@ class Context:
         return n.value, ms.value
 
     def plane_variant(self, bits: int = 32) -> int:
-        """V_loc plane kernel chosen at setup for the given arithmetic (32, 64 or 48 = double-float)."""
+        """V_loc plane kernel chosen at setup for the given arithmetic (32, 64 or 48 = double-float).
+
+        The numbers are those of wdf_plane_variant (include/wdf.h); 6 is the line-resident kernel (8)
+        on 64 x 64 double-float planes whose band it takes.
+        """
         v = ctypes.c_int()
         self._check(self._lib.wdf_plane_variant(self._ctx, int(bits), ctypes.byref(v)))
         return v.value
