@@ -94,15 +94,15 @@ ALU_PEAK_SOURCE = {"mixed_df": "FP32: 152 SMs x 128 lanes x 2 flop x 2070 MHz (d
                    "fp64": "FP64: measured FMA loop on GB300, 1.19 TFLOP/s"}
 
 
-# DRAM bytes per (pair, z plane) unit of the FP32 V_loc plane kernel, per (grid, kernel variant
-# chosen at setup), from one ncu capture each on a small case of the same system
-# (dram__bytes_read.sum + dram__bytes_write.sum over the units of the captured launch; see
-# profiles/); traffic grows in proportion to the units launched. The 64 value is that of the kernel's earlier form,
-# which copied the same slices. A variant without a capture reports null.
+# DRAM bytes per (pair, z plane) unit of the FP32 V_loc plane kernel, per (grid, largest |n1| of the
+# sphere, kernel variant chosen at setup), from one ncu capture each (dram__bytes_read.sum +
+# dram__bytes_write.sum over the units of the captured launch; see profiles/); traffic grows in
+# proportion to the units launched. A sphere or variant without a capture of its present kernel
+# reports null.
 PLANE_DRAM_BYTES_PER_UNIT = {
-    (64, 1): (210.873088e6 + 167.385088e6) / 32768,  # k_plane_reg<64>: 32,768 units
-    (64, 5): (210.877440e6 + 149.595648e6) / 32768,  # k_plane_pipe<64, 15>: 32,768 units
-    (96, 5): (157.77e6 + 95.63e6) / 12288,  # k_plane_pipe<96, 22>: 12,288 units
+    (64, 15, 1): (210.873088e6 + 167.385088e6) / 32768,  # k_plane_reg<64>: 32,768 units
+    (64, 15, 5): (210.849e6 + 146.837e6) / 32768,  # k_plane_pipe<64, 15>: 32,768 units
+    (96, 22, 5): (157.77e6 + 95.63e6) / 12288,  # k_plane_pipe<96, 22>: 12,288 units
 }
 
 
@@ -290,7 +290,8 @@ def roofline_line(s, precision, variant, k_launches, k_ms, k_blocks, steps, ms_d
     full = np.concatenate([s.miller, -s.miller[1:]])
     ndisk = len({(int(a), int(b)) for a, b, _ in full})
     alg_bytes = blocks_per_launch * 2 * ndisk * 8
-    per_unit = PLANE_DRAM_BYTES_PER_UNIT.get((s.grid[0], variant)) if precision != "fp64" else None
+    xmax = int(np.abs(s.miller[:, 0]).max())
+    per_unit = PLANE_DRAM_BYTES_PER_UNIT.get((s.grid[0], xmax, variant)) if precision != "fp64" else None
     return {"kernel": target, "variant": variant, "bound": bound, "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s",
             "frac": (achieved / alu_peak) if achieved else None, "traffic": per_unit * blocks_per_launch if per_unit else None,
             "traffic_unit": "bytes per launch (DRAM read + write, ncu)", "algorithmic_bytes_per_launch": alg_bytes,
