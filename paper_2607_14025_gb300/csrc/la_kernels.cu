@@ -547,8 +547,8 @@ __global__ void __launch_bounds__(256) k_lincomb(Geo g, cplx<T> *__restrict__ Y,
 // FP64 linear combinations: a warp owns 32 elements (a block LE = 128) of VQ
 // vectors, each lane one element, rows of U read once per VQ vectors (coalesced, from L2), the
 // scaled coefficients staged LJ64 rows at a time. As for the Gram products only the FMAs count: at
-// most VQ - 1 padded vectors and enough blocks for the 152 SMs. VQ = 4 until the vectors alone
-// make two blocks per SM with 8. Against the 128 x 32 tile of k_lincomb: 42 rows into 56 vectors of
+// most VQ - 1 padded vectors and enough blocks for the 152 SMs. One and two vectors have their own VQ, else
+// VQ = 4, and 8 once that still leaves four blocks per SM. Against the 128 x 32 tile of k_lincomb: 42 rows into 56 vectors of
 // 1,800 elements 97 -> 20 us, 128 rows into 48 of 8,455 278 -> 201 us, 64 into 47 138 -> 101 us.
 constexpr int LJ64 = 64;
 

@@ -10,12 +10,15 @@
 // factors), powers by Cooley-Tukey with constant twiddles. The power-of-two factor comes first in
 // the inverse and last in the forward transform, where the zero inputs and dead outputs are.
 //
-// Double-float sums stay unnormalised inside a transform: the low part grows to a few ulp of the
-// high part, which the next TwoSum of the leading parts absorbs (8 FP32 operations a sum instead of
-// 11, 4 a product instead of 7); the caller renormalises what it stores.
+// Double-float sums stay unnormalised inside a transform: 8 FP32 operations a sum instead of 11, 4 a
+// product instead of 7; the caller renormalises what it stores. With u = 2^-24 and A the sum of the
+// inputs' magnitudes, the low part after k steps in a row is at most (k + 1) u A (each step adds a
+// rounding error of the leading parts, u A at most), so a step's own rounding, of the low parts, is at most
+// 2 (k + 1) u^2 A and that of the whole transform about k^2 u^2 A: k is at most 15 for the 32 points a lane
+// holds, 8e-13 A if every rounding went one way. Measured against 64-bit arithmetic, A_v x on 96^3 is off
+// by 4.1e-15 and on 64^3 by 3.2e-15 of its largest component, as with sums renormalised throughout.
 #pragma once
 
-#include <cstring>
 #include <utility>
 
 #include "common.cuh"
@@ -106,10 +109,7 @@ template <typename T> struct CA {
 struct pdf {
   u64 h, l;
 };
-#ifdef __CUDACC__
 static __constant__ u64 kNegZero2 = 0x8000000080000000ull;
-#endif
-#ifdef __CUDA_ARCH__
 __device__ __forceinline__ u64 pk(float a, float b) {
   u64 r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
@@ -141,23 +141,6 @@ __device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
 __device__ __forceinline__ u64 mul2(u64 a, u64 b) {
   return fma2(a, b, kNegZero2);
 }
-#else  // the same operations for the host pass (the arithmetic tests on the CPU)
-inline u64 pk(float a, float b) {
-  u64 r;
-  float v[2] = {a, b};
-  memcpy(&r, v, 8);
-  return r;
-}
-inline float2 upk(u64 a) {
-  float2 v;
-  memcpy(&v, &a, 8);
-  return v;
-}
-inline u64 add2(u64 a, u64 b) { return pk(upk(a).x + upk(b).x, upk(a).y + upk(b).y); }
-inline u64 sub2(u64 a, u64 b) { return pk(upk(a).x - upk(b).x, upk(a).y - upk(b).y); }
-inline u64 mul2(u64 a, u64 b) { return pk(upk(a).x * upk(b).x, upk(a).y * upk(b).y); }
-inline u64 fma2(u64 a, u64 b, u64 c) { return pk(fmaf(upk(a).x, upk(b).x, upk(c).x), fmaf(upk(a).y, upk(b).y, upk(c).y)); }
-#endif
 
 // FP32 complex numbers as one packed pair: a complex sum is one instruction, a product by a constant
 // or a twiddle two. The FP32 pipe takes as long as for the scalar pairs, but half of the issue slots go to
@@ -178,13 +161,9 @@ template <> struct CA<float> {
   static __device__ __forceinline__ C sub(C a, C b) { return sub2(a, b); }
   static __device__ __forceinline__ C neg(C a) { return pmul(a, both(-1.0)); }
   static __device__ __forceinline__ C pmul(C a, C b) {
-#ifdef __CUDA_ARCH__
     u64 r;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
-#else
-    return mul2(a, b);
-#endif
   }
   template <int S> static __device__ __forceinline__ C muli(C a) { return pmul(swap(a), alt(S)); }
   template <int S> static __device__ __forceinline__ C addi(C a, C b) { return fma2(swap(b), alt(S), a); }
@@ -325,8 +304,7 @@ template <int I, int E, typename F> __device__ __forceinline__ void static_for(F
   }
 }
 
-constexpr u64 all_of(int n) { return n >= 64 ? ~0ull : (1ull << n) - 1; }
-// masks longer than 64 inputs are built from a predicate on the index instead (band_mask)
+// masks of the inputs that can be non-zero: a predicate on the index
 struct Full {
   static constexpr bool at(int) { return true; }
 };

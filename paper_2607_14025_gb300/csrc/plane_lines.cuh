@@ -30,7 +30,10 @@ namespace wdf {
 
 // lanes per line, planes and warps per block, blocks per SM the registers are bounded for, chunks
 // of the exchange. Registers: 2 N (FP32) or 4 M (double-float) hold the line. Shared memory: one
-// plane's tile is N (2 (N / 4) + 1) values.
+// plane's tile is N (2 (N / 4) + 1) values. L is the fewest lanes that divide their own share of the
+// line (L | N / L) with at most 80 points a lane in FP32 and 30 in double-float and FP64; C keeps the
+// exchange at 10 values or fewer per lane and chunk (12 in FP32); B is what the registers and
+// the tiles leave.
 template <typename T, int N> struct Lines {
   static constexpr int L = 0, P = 1, W = 1, B = 1, C = 1;  // L = 0: no instance
 };

@@ -498,7 +498,8 @@ void launch_tc_prep_u(const Geo &g, const float2 *U, int na, float *uwh, float *
   WDF_CUDA_TRY(cudaGetLastError());
 }
 
-// K splits of the Gram: one CTA per SM (shared memory), so the launch runs in waves of nsm CTAs;
+// K splits of the Gram: one CTA per SM at a time (each takes all 512 TMEM columns), so the launch runs in
+// waves of nsm CTAs;
 // choose the split count (at most nch / 4, so that each CTA fills its four stages) that minimises
 // waves x (chunks per CTA + 12) + sums, the 12 standing for a CTA's partial-sum write (128 x 192
 // doubles, about the bytes of two dozen 16-value X chunks, written without waiting) and the sums for
