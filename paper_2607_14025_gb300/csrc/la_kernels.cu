@@ -919,7 +919,8 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
   typedef typename UpdVec<T>::K KV;
   constexpr int E = UpdVec<T>::E, UB = 2, STEP = 256 * E * UB;
   const int i = blockIdx.x, c = blockIdx.y;
-  __shared__ double redp[8], red3[3][8], fold[3][256];
+  __shared__ double redp[8], red3[3][8];
+  extern __shared__ __align__(8) double fold[];  // 3 x 256 where an FP32 solve's block takes more than DCHUNK elements
   pdl_begin();
   pdl_wait();
   if (i == 0 && c == 0 && threadIdx.x == 0) s.nactive[which ^ 1] = 0;  // the next launch's count
@@ -963,8 +964,9 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
   // a thread's sums over DCHUNK elements of the row are FP32 in an FP32 solve; a block that takes more adds them
   // up in FP64 (in shared memory: the registers are all in use)
   A vrz = 0, vrr = 0, vr3 = 0;
+  constexpr bool F32 = std::is_same<A, float>::value;
   const int t = threadIdx.x;
-  const bool more = e + DCHUNK < e1;
+  const bool more = F32 && e + DCHUNK < e1;
   for (; e < e1; e += STEP, load(e)) {
 #pragma unroll
     for (int u = 0; u < UB; ++u) {
@@ -1001,17 +1003,17 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(Geo g, cplx<T> *__restrict
     }
     if (more && (e & (DCHUNK - 1)) >= DCHUNK - STEP && e + STEP < e1) {  // e0 is a multiple of DCHUNK
       const bool first = e - e0 < DCHUNK;
-      fold[0][t] = first ? cast<double>(vrz) : fold[0][t] + cast<double>(vrz);
-      fold[1][t] = first ? cast<double>(vrr) : fold[1][t] + cast<double>(vrr);
-      if (fb) fold[2][t] = first ? cast<double>(vr3) : fold[2][t] + cast<double>(vr3);
+      fold[t] = first ? cast<double>(vrz) : fold[t] + cast<double>(vrz);
+      fold[256 + t] = first ? cast<double>(vrr) : fold[256 + t] + cast<double>(vrr);
+      if (fb) fold[512 + t] = first ? cast<double>(vr3) : fold[512 + t] + cast<double>(vr3);
       vrz = vrr = vr3 = 0;
     }
   }
   double sum[3] = {cast<double>(vrz), cast<double>(vrr), fb ? cast<double>(vr3) : 0.0};
   if (more) {
-    sum[0] += fold[0][t];
-    sum[1] += fold[1][t];
-    if (fb) sum[2] += fold[2][t];
+    sum[0] += fold[t];
+    sum[1] += fold[256 + t];
+    if (fb) sum[2] += fold[512 + t];
   }
   block_sum3(sum, fb, red3);
   if (threadIdx.x != 0) return;
@@ -1061,7 +1063,8 @@ void launch_cg_update(const Geo &g, cplx<T> *x, cplx<T> *r, const cplx<T> *p, co
   // 152 SMs twice over, so that a block's start and sums weigh less
   const int chunk = (long)n * ((g.nint + 4 * DCHUNK - 1) / (4 * DCHUNK)) >= 8 * 152 ? 4 * DCHUNK : DCHUNK;
   const int nchunk = (g.nint + chunk - 1) / chunk;
-  launch_pdl("cg_update", bits_of<T>(), (long long)n * nchunk, k_cg_update<T>, dim3(n, nchunk), dim3(256), 0, st, g, x, r, p, Ap, kprec, s, nchunk, chunk, dots, ndot,
+  const size_t sm = std::is_same<T, float>::value && chunk > DCHUNK ? 3 * 256 * sizeof(double) : 0;
+  launch_pdl("cg_update", bits_of<T>(), (long long)n * nchunk, k_cg_update<T>, dim3(n, nchunk), dim3(256), sm, st, g, x, r, p, Ap, kprec, s, nchunk, chunk, dots, ndot,
          maxiter, which);
   WDF_CUDA_TRY(cudaGetLastError());
 }
