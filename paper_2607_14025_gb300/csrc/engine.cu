@@ -821,20 +821,20 @@ void sternheimer_solve(wdf_ctx *c, const cplx<double> *b, cplx<double> *x, const
 // Orbitals whose real-space fields (one perturbation pair's, `real` bytes a real number) are held at once in the
 // density response, and the buffer: psi = 1 on the grid first, the fields `head` bytes on. The
 // refinement's A x (two rows per pair and orbital) is idle by then and holds one orbital's fields in 15 for each
-// pair (a row is a 31st of the grid on the model spheres): all of them from 16 pairs on. Blocks of
-// few solves have a buffer of their own of at most 64 MB. Memory that cannot be had is no error: 0 means the kernels that sum in place, which need
+// pair (a row is a 31st of the grid on the model spheres): all of them from 16 pairs on. Where a
+// buffer of their own of at most 64 MB holds more, that one is used (48^3, 32 orbitals, 12 pairs: one
+// group instead of two, 0.4% of the call). Memory that cannot be had is no error: 0 means the kernels that sum in place, which need
 // none (64 orbitals on 64^3, 2,048 solves: 4.5 ms against 3.0). Under a limit on the library's memory
 // the buffer is given back at once. (With all fields in a buffer of their own, 268 MB for those 64 orbitals,
 // calls were refused under limits that had been enough for the sum in place.)
 static int orbital_group(wdf_ctx *c, size_t real, DBuf **space, size_t &head) {
-  constexpr int kFew = 8;
   constexpr size_t kOwnBytes = (size_t)64 << 20;
   const size_t field = 2 * real * c->ngrid;
   head = (real * c->ngrid + 255) / 256 * 256;
   auto room = [&](size_t bytes) { return bytes > head ? (int)std::min<size_t>(c->nocc, (bytes - head) / field) : 0; };
   int group = room(c->rAx.cap);
   *space = &c->rAx;
-  if (group < std::min(c->nocc, kFew)) {
+  if (group < c->nocc) {
     const int own = std::min(c->nocc, std::max(1, room(kOwnBytes)));
     if (own > group && c->orbfields.try_ensure(head + field * own)) {
       group = own;
